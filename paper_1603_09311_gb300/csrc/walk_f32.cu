@@ -31,6 +31,23 @@ namespace sdd {
 __device__ __forceinline__ float one_plus(uint32_t w) { return mant_one(w); }
 __device__ __forceinline__ float uni23(uint32_t w) { return one_plus(w) - 0.99999994039535522f; }
 
+// |x| and -x as sign bits alone.  Under -ftz=true fabsf() and unary minus
+// flush denormals, which the compiler forms as an addition of their own; the
+// float operations that take these flush their inputs anyway, so the plain
+// forms give the same results as operand modifiers, without an instruction.
+// There were four such additions a step (of about 62 issue slots): the squared
+// radius, its negated root and the two coordinates of the wall distance.
+__device__ __forceinline__ float abs_bits(float x) {
+    float r;
+    asm("abs.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float neg_bits(float x) {
+    float r;
+    asm("neg.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // Occupation counters.  KMAX = 2: the step count of material 1.  KMAX = 3, 4:
 // power sums s_p = sum over steps of m^p (p = 1 .. KMAX-1), which determine
 // the counts of materials 1 .. KMAX-1 (a Vandermonde system, solved once at
@@ -327,7 +344,7 @@ struct WalkerF32 {
     __device__ __forceinline__ static Incr increment(const WalkArgs &A, uint32_t wa, uint32_t wb) {
         Incr d;
         // |.| only guards the last-ulp sign of lg2 near u0 = 1
-        d.r = sqrtf(fabsf(A.f_cdt * __log2f(uni23(wa))));
+        d.r = sqrtf(abs_bits(A.f_cdt * __log2f(uni23(wa))));
         __sincosf(fmaf(one_plus(wb), 6.28318530718f, -9.42477796077f), &d.sn, &d.cs);
         return d;
     }
@@ -338,9 +355,10 @@ struct WalkerF32 {
     // when the walk reached the boundary.
     __device__ __forceinline__ bool advance(const ModelDev &M, const WalkArgs &A, const Incr &d,
                                             uint32_t wa, uint32_t wb, uint32_t k, ExitInfo<float> &ei) {
-        const float Xn = fmaf(-d.r, d.cs, X);
-        const float Zn = fmaf(-d.r, d.sn, Z);
-        const float dn = fminf(M.fhw - fabsf(Xn), M.fhh - fabsf(Zn));
+        const float nr = neg_bits(d.r);
+        const float Xn = fmaf(nr, d.cs, X);
+        const float Zn = fmaf(nr, d.sn, Z);
+        const float dn = fminf(M.fhw - abs_bits(Xn), M.fhh - abs_bits(Zn));
         const float pn = dmin * dn;
         if (pn <= A.f_bthr) {
             if (near_wall(M, A, Xn, Zn, dn, pn, wa, wb, ei)) {
@@ -384,9 +402,10 @@ struct WalkerF32 {
     __device__ __forceinline__ bool advance_cell(const ModelDev &M, const WalkArgs &A, const Incr &d,
                                                  uint32_t wa, uint32_t wb, uint32_t k, ExitInfo<float> &ei,
                                                  uint32_t &ci, uint32_t &off) {
-        const float Xn = fmaf(-d.r, d.cs, X);
-        const float Zn = fmaf(-d.r, d.sn, Z);
-        const float dn = fminf(M.fhw - fabsf(Xn), M.fhh - fabsf(Zn));
+        const float nr = neg_bits(d.r);
+        const float Xn = fmaf(nr, d.cs, X);
+        const float Zn = fmaf(nr, d.sn, Z);
+        const float dn = fminf(M.fhw - abs_bits(Xn), M.fhh - abs_bits(Zn));
         const float pn = dmin * dn;
         if (pn <= A.f_bthr) {
             if (near_wall(M, A, Xn, Zn, dn, pn, wa, wb, ei)) {
