@@ -759,7 +759,9 @@ sdd_status sdd_model_program(const sdd_model_desc *model, int32_t *program, int3
  *   n_paths [n_nodes] host; warps >= 1; guided_factor >= 1 (guided items of
  *   about 1 / (guided_factor x warps) of the paths not yet cut, multiples of
  *   32 shrinking toward the end of the queue) used when chunk_paths == 0,
- *   else fixed items of chunk_paths paths, node by node.
+ *   else fixed items of chunk_paths paths, node by node.  (Single-precision TE
+ *   calls of at most 16 walks a warp are cut into items of one share each
+ *   instead, node by node: the cooperative rounds of the walk take those.)
  *   node, path0, count [max_items] host, written in queue order; *n_items
  *   the number of items.
  * Errors: SDD_E_ARG for n_nodes < 0, a negative path count, warps < 1,

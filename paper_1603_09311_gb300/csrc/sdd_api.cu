@@ -496,7 +496,20 @@ struct Launch {
     int chunk;   // > 0: fixed items of chunk paths; 0: guided
     int factor;  // guided: an item takes about 1 / (factor x warps) of the queued paths
     int64_t max_steps;
+    bool coop;   // the walk has cooperative rounds
 };
+
+// Walks a warp takes at a time.  32, one a lane, unless the call has so few
+// walks that every warp of the grid can take its share of them in cooperative
+// rounds: then that share (and items of that size), so that all warps work.
+// One node x 1000 walks at dt 1e-3 took 0.157 ms with one warp for 32 walks
+// and 0.040 ms with a warp for each; 16000 walks 0.172 and 0.080 ms, 32000
+// 0.175 and 0.115 ms.  Above kCoopWalks a warp fills its lanes.
+int warp_lanes(long long total, const Launch &L) {
+    const long long W = std::max<long long>(1, (long long)L.grid * (L.block / 32));
+    const long long share = (total + W - 1) / W;
+    return L.coop && L.chunk == 0 && share <= kCoopWalks ? (int)std::max<long long>(share, 1) : 32;
+}
 
 // Key of a launch shape in the tuning cache file: device, lookup program,
 // materials bound, evaluations, precision and the decade of dt.
@@ -549,6 +562,7 @@ Launch choose_launch(const sdd_ctx *ctx, const sdd_config *cfg, double dt,
     L.chunk = (cfg && cfg->chunk_paths) ? cfg->chunk_paths : 0;
     L.max_steps = (cfg && cfg->max_steps) ? cfg->max_steps : (int64_t)std::ceil(20.0 / dt);
     if (L.max_steps > kMaxSteps) L.max_steps = kMaxSteps;
+    L.coop = !L.f64 && gcode != GC_TM;
     L.max_steps = (L.max_steps + 7) / 8 * 8;  // single-precision walks advance 8 steps per iteration
     return L;
 }
@@ -633,14 +647,16 @@ Plan plan_work(int32_t n_nodes, const int64_t *begin, const int64_t *count, uint
     P.node_item0.assign((size_t)n_nodes + 1, 0);
     for (int j = 0; j < n_nodes; ++j) P.total_paths += count[j];
     auto first = [&](int j) -> int64_t { return begin ? begin[j] : 0; };
-    if (L.chunk > 0) {
+    const int lanes = warp_lanes(P.total_paths, L);
+    if (L.chunk > 0 || lanes < 32) {
+        const int chunk = L.chunk > 0 ? L.chunk : lanes;
         for (int j = 0; j < n_nodes; ++j) {
             P.node_item0[j] = (int32_t)P.items.size();
-            for (int64_t p = 0; p < count[j]; p += L.chunk) {
+            for (int64_t p = 0; p < count[j]; p += chunk) {
                 Item I;
                 I.node = j;
                 I.path0 = p_offset + (uint32_t)(first(j) + p);
-                I.count = (int32_t)std::min<int64_t>(L.chunk, count[j] - p);
+                I.count = (int32_t)std::min<int64_t>(chunk, count[j] - p);
                 I.model = 0;
                 P.items.push_back(I);
             }
@@ -737,9 +753,12 @@ const Plan &plan_cached(sdd_ctx *ctx, int32_t n_nodes, const int64_t *n_paths, u
                         const Launch &L) {
     PlanKey key;
     key.paths.assign(n_paths, n_paths + n_nodes);
-    key.chunk = L.chunk;
-    key.factor = L.chunk > 0 ? 0 : L.factor;
-    key.warps = L.chunk > 0 ? 0 : (long long)L.grid * (L.block / 32);
+    long long total = 0;
+    for (int j = 0; j < n_nodes; ++j) total += n_paths[j];
+    const int lanes = warp_lanes(total, L);
+    key.chunk = lanes < 32 ? lanes : L.chunk;
+    key.factor = key.chunk > 0 ? 0 : L.factor;
+    key.warps = key.chunk > 0 ? 0 : (long long)L.grid * (L.block / 32);
     key.offset = p_offset;
     if (ctx->plan_valid && key == ctx->plan_key) {
         ctx->plan.cached = true;
@@ -770,6 +789,17 @@ WalkArgs base_args(sdd_ctx *ctx, const Launch &L, double dt, uint64_t seed) {
         A.rk1[r] = A.key1 + (uint32_t)r * 0xBB67AE85u;
     }
     A.max_steps = (uint32_t)L.max_steps;
+    A.max_lanes = 32;
+    // Recording an ended walk and refilling its lane costs the warp about 300
+    // instructions, however many lanes take part; a lane that waits idles.
+    // The best batch goes with the square root of the ended walks per step:
+    // measured optima at 150, 290, 970 steps a walk were 6, 4, 3 (dt 2e-3,
+    // 1e-3, 3e-4: 8.02 -> 6.92, 14.98 -> 14.07, 8.45 -> 8.18 ms against one at
+    // a time), none at 2900.  A walk takes about the domain's slowest decay
+    // time.
+    const double wx = 2.0 * ctx->M.hw, wz = 2.0 * ctx->M.hh;
+    const double len = 2.0 / (9.8696 * (1.0 / (wx * wx) + 1.0 / (wz * wz))) / dt;
+    A.exit_batch = (int32_t)std::min(6.0, std::max(1.0, std::floor(75.0 / std::sqrt(len) + 0.5)));
     return A;
 }
 
@@ -851,6 +881,7 @@ sdd_status enqueue(sdd_ctx *ctx, const Plan &P, const Launch &L, WalkArgs A, cud
     SDD_CUDA(cudaMemsetAsync(ctx->counters.p, 0, 3 * sizeof(unsigned long long), s));
     A.items = (const Item *)ctx->items.p;
     A.n_items = (int32_t)ni;
+    A.max_lanes = P.qbase.empty() ? warp_lanes(P.total_paths, L) : 32;
     table_args(P, n_nodes, reinterpret_cast<const unsigned char *>(ctx->items.p), A);
     A.slots = (double *)ctx->slots.p;
     A.item_trunc = (int32_t *)ctx->trunc.p;
@@ -1753,6 +1784,7 @@ extern "C" sdd_status sdd_interface_values_async(sdd_ctx *ctx, const double *nod
         A.node_ids = node_ids ? reinterpret_cast<const uint32_t *>(r->dev + o_ids) : nullptr;
         A.items = reinterpret_cast<const Item *>(r->dev + o_items);
         A.n_items = (int32_t)ni;
+        A.max_lanes = warp_lanes(P.total_paths, L);
         A.order = P.order.empty() ? nullptr : reinterpret_cast<const int32_t *>(r->dev + o_order);
         A.slots = reinterpret_cast<double *>(r->dev + o_slots);
         A.item_trunc = reinterpret_cast<int32_t *>(r->dev + o_trunc);

@@ -158,6 +158,15 @@ struct WalkerF32 {
     uint32_t nid, pre_x, pre_y;
     const uint32_t *tco;  // GC_RASTER_MULTI: the tile map of this walk's model
 
+    // Shared address of the lane's column of WarpSmem::pend: the step that
+    // ends a walk puts there the point before it, its proposed point, its
+    // bridge uniform (negative: it overshot a wall) and its number.
+    // finalize() turns them into the exit record, for all ended lanes of the
+    // warp at once.  Through shared memory, not registers: the eight exits of
+    // an unrolled iteration then leave nothing but the lane's state to merge
+    // (in registers it cost 4.6 issue slots a step in moves).
+    uint32_t pend;
+
     __device__ __forceinline__ static bool in_rect(const ShapeDev &S, float X, float Z) {
         return X >= S.f[0] && X < S.f[1] && Z >= S.f[2] && Z < S.f[3];
     }
@@ -245,6 +254,12 @@ struct WalkerF32 {
         }
     }
 
+    // The accepted step at (x, z) into the occupation counters.
+    __device__ __forceinline__ void count_step(const ModelDev &M, float x, float z) {
+        if constexpr (kRegions) count_regions(M, x, z);
+        else occ.add(material(M, x, z));
+    }
+
     // Counts of materials 1 .. KMAX-1 after nocc counted steps.  Region
     // counters: the shape has cs; with the shape in the earth the earth
     // background has ce - cs and the air nocc - ce, with the shape in the air
@@ -262,7 +277,11 @@ struct WalkerF32 {
             occ.counts(c);
         }
     }
-    __device__ __forceinline__ void bind(HistT *h) { occ.bind((uint32_t)__cvta_generic_to_shared(h)); }
+    __device__ __forceinline__ void bind(HistT *h, float *p) {
+        occ.bind((uint32_t)__cvta_generic_to_shared(h));
+        pend = (uint32_t)__cvta_generic_to_shared(p);
+    }
+    static constexpr int kPend = 6;
 
     __device__ __forceinline__ void start(const ModelDev &M, const WalkArgs &A, double x0,
                                           double z0, uint32_t path, uint32_t node_id, int model) {
@@ -277,8 +296,19 @@ struct WalkerF32 {
         pre_y = 0xCD9E8D57u * node_id;
     }
 
-    __device__ __forceinline__ void place(const ModelDev &M, float Xn, float Zn, float th, int w,
-                                          ExitInfo<float> &ei) const {
+    __device__ __forceinline__ void put_exit(float X0, float Z0, float Xn, float Zn, float U, uint32_t k) const {
+        asm volatile("st.shared.f32 [%0], %1;\n\tst.shared.f32 [%0+128], %2;\n\tst.shared.f32 [%0+256], %3;\n\t"
+                     "st.shared.f32 [%0+384], %4;\n\tst.shared.f32 [%0+512], %5;\n\tst.shared.u32 [%0+640], %6;"
+                     ::"r"(pend), "f"(X0), "f"(Z0), "f"(Xn), "f"(Zn), "f"(U), "r"(k) : "memory");
+    }
+    __device__ __forceinline__ void get_exit(float &X0, float &Z0, float &Xn, float &Zn, float &U, uint32_t &k) const {
+        asm volatile("ld.shared.f32 %0, [%6];\n\tld.shared.f32 %1, [%6+128];\n\tld.shared.f32 %2, [%6+256];\n\t"
+                     "ld.shared.f32 %3, [%6+384];\n\tld.shared.f32 %4, [%6+512];\n\tld.shared.u32 %5, [%6+640];"
+                     : "=f"(X0), "=f"(Z0), "=f"(Xn), "=f"(Zn), "=f"(U), "=r"(k) : "r"(pend) : "memory");
+    }
+
+    __device__ __forceinline__ static void place(const ModelDev &M, float X, float Z, float Xn, float Zn, float th,
+                                                 int w, ExitInfo<float> &ei) {
         ei.th = th;
         ei.wall = w;
         ei.x = fmaf(th, Xn - X, X);
@@ -287,51 +317,70 @@ struct WalkerF32 {
         if (w == 1) ei.x = M.fhw;
         if (w == 2) ei.z = -M.fhh;
         if (w == 3) ei.z = M.fhh;
-        ei.mlast = material(M, X, Z);
     }
 
-    // The step (X, Z) -> (Xn, Zn) came within reach of a wall (rare; taken by
-    // few lanes of a warp at a time, so kept short).  Overshoot (dn <= 0):
-    // theta_w = d_w / (d_w - d'_w) over the walls with d'_w <= 0, smallest
-    // first, ties to the first of left, right, top, bottom.  Both inside: the
+    // Whether the step (X, Z) -> (Xn, Zn), which came within reach of a wall,
+    // ends the walk.  Overshoot (dn <= 0): yes.  Both ends inside: the
     // Brownian-bridge test with one uniform for all walls: the walk touched a
     // wall iff 2 d_w d'_w / dt <= -ln U for the smallest product, tested as
     // U <= exp(-2 d_w d'_w / dt).  U is made of the 18 bits of the step's two
     // Philox words that the normals leave unused:
-    // U = (high 9 bits of wa : high 9 bits of wb + 1/2) 2^-18.  Every
-    // product d_w d'_w is at least pn = dmin dn (the nearest distances before
-    // and after the step), so U > exp(-2 pn / dt) rules out a hit without
-    // forming the four products; most near-wall steps end there.
-    __device__ __forceinline__ bool near_wall(const ModelDev &M, const WalkArgs &A, float Xn,
-                                              float Zn, float dn, float pn, uint32_t wa, uint32_t wb,
-                                              ExitInfo<float> &ei) const {
-        const float d[4] = {X + M.fhw, M.fhw - X, Z + M.fhh, M.fhh - Z};
-        const float e[4] = {Xn + M.fhw, M.fhw - Xn, Zn + M.fhh, M.fhh - Zn};
-        const uint32_t u18 = ((wa >> 23) << 9) | (wb >> 23);
-        const float U = fmaf((float)u18, 3.814697265625e-06f, 1.9073486328125e-06f);
+    // U = (high 9 bits of wa : high 9 bits of wb + 1/2) 2^-18, here as the
+    // mantissa of a float in [1, 2) less 1 - 2^-19 (exact).  Every product
+    // d_w d'_w is at least pn = dmin dn (the nearest distances before and
+    // after the step), so U > exp(-2 pn / dt) rules out a hit without forming
+    // the distances; most near-wall steps end there.
+    //
+    // A warp takes this branch on about every second step (one lane of 32 is
+    // enough), and the code stands once per unrolled step: it holds the
+    // decision alone.  What follows a hit (the wall, theta, the exit point,
+    // the last material) waits for finalize().
+    __device__ __forceinline__ static bool reaches_wall(const ModelDev &M, const WalkArgs &A, float X0,
+                                                        float Z0, float Xn, float Zn, float dn, float pn,
+                                                        uint32_t wa, uint32_t wb, float &U) {
+        U = __uint_as_float(0x3f800000u | ((wa >> 9) & 0x7fc000u) | ((wb >> 18) & 0x3fe0u)) - 0.99999809265136719f;
         if (dn > 0.f && U > __expf(-pn * A.f_c2dt)) return false;
-        if (dn <= 0.f) {
+        const float p0 = (X0 + M.fhw) * (Xn + M.fhw), p1 = (M.fhw - X0) * (M.fhw - Xn);
+        const float p2 = (Z0 + M.fhh) * (Zn + M.fhh), p3 = (M.fhh - Z0) * (M.fhh - Zn);
+        const float pmin = fminf(fminf(p0, p1), fminf(p2, p3));
+        const bool hit = dn <= 0.f || !(U > __expf(-(pmin * A.f_c2dt)));
+        U = dn <= 0.f ? -1.f : U;
+        return hit;
+    }
+
+    // The exit record of an ended walk (st: 1 reached the boundary,
+    // 2 truncated).  Overshoot: theta_w = d_w / (d_w - d'_w) over the walls
+    // with d'_w <= 0, smallest first, ties to the first of left, right, top,
+    // bottom.  Bridge hit: the wall of the smallest product (first in wall
+    // order) and theta = (2 d d' / dt) / (-ln U).
+    __device__ __forceinline__ void finalize(const ModelDev &M, const WalkArgs &A, int st, ExitInfo<float> &ei) const {
+        float X, Z, pXn, pZn, pU;
+        get_exit(X, Z, pXn, pZn, pU, ei.nocc);
+        if (st == 2) {
+            ei.x = X; ei.z = Z; ei.th = 0.f; ei.wall = 0;
+        } else {
+            const float d[4] = {X + M.fhw, M.fhw - X, Z + M.fhh, M.fhh - Z};
+            const float e[4] = {pXn + M.fhw, M.fhw - pXn, pZn + M.fhh, M.fhh - pZn};
             float best = 2.0f;
             int bw = 0;
+            if (pU < 0.f) {
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                if (e[w] <= 0.f) {
-                    const float t = d[w] / (d[w] - e[w]);
-                    if (t < best) { best = t; bw = w; }
+                for (int w = 0; w < 4; ++w) {
+                    if (e[w] <= 0.f) {
+                        const float t = d[w] / (d[w] - e[w]);
+                        if (t < best) { best = t; bw = w; }
+                    }
                 }
+            } else {
+                const float p0 = d[0] * e[0], p1 = d[1] * e[1], p2 = d[2] * e[2], p3 = d[3] * e[3];
+                const float pmin = fminf(fminf(p0, p1), fminf(p2, p3));
+                const float es = pmin * A.f_c2dt;
+                bw = p0 == pmin ? 0 : (p1 == pmin ? 1 : (p2 == pmin ? 2 : 3));
+                best = es / -logf(pU);
             }
-            place(M, Xn, Zn, best, bw, ei);
-            return true;
+            place(M, X, Z, pXn, pZn, best, bw, ei);
         }
-        const float p0 = d[0] * e[0], p1 = d[1] * e[1], p2 = d[2] * e[2], p3 = d[3] * e[3];
-        const float pmin = fminf(fminf(p0, p1), fminf(p2, p3));
-        const float es = pmin * A.f_c2dt;
-        if (U > __expf(-es)) return false;
-        // a hit: the wall of the smallest product (first in wall order) and
-        // the fraction theta = (2 d d' / dt) / (-ln U)
-        const int bw = p0 == pmin ? 0 : (p1 == pmin ? 1 : (p2 == pmin ? 2 : 3));
-        place(M, Xn, Zn, es / -logf(U), bw, ei);
-        return true;
+        ei.mlast = material(M, X, Z);
     }
 
     // The part of an Euler step that does not depend on the position: the
@@ -349,34 +398,39 @@ struct WalkerF32 {
         return d;
     }
 
-    // The rest of the step: move, test the walls, count the occupation.
-    // Only the high 9 bits of wa and wb are read (the bridge uniform, on the
-    // rare steps near a wall).  k = steps of this walk since n.  Returns true
-    // when the walk reached the boundary.
-    __device__ __forceinline__ bool advance(const ModelDev &M, const WalkArgs &A, const Incr &d,
-                                            uint32_t wa, uint32_t wb, uint32_t k, ExitInfo<float> &ei) {
-        const float nr = neg_bits(d.r);
-        const float Xn = fmaf(nr, d.cs, X);
-        const float Zn = fmaf(nr, d.sn, Z);
-        const float dn = fminf(M.fhw - abs_bits(Xn), M.fhh - abs_bits(Zn));
-        const float pn = dmin * dn;
-        if (pn <= A.f_bthr) {
-            if (near_wall(M, A, Xn, Zn, dn, pn, wa, wb, ei)) {
-                ei.nocc = n + k;
+    // The rest of two steps (Philox words w): the moves, one branch for both
+    // wall tests, the occupation.  k: steps of this walk since n.  Returns
+    // true when the walk reached the boundary.  The branch and its
+    // reconvergence cost three issue slots; one for two steps took 64 nodes x
+    // 1e5 walks, dt 1e-4, from 41.4 to 40.3 ms (one for four or for eight:
+    // 42.8 and 42.3 ms, more live positions).
+    __device__ __forceinline__ bool advance2(const ModelDev &M, const WalkArgs &A, const uint4 &w, uint32_t k) {
+        const Incr a = increment(A, w.x, w.y), b = increment(A, w.z, w.w);
+        const float ra = neg_bits(a.r), rb = neg_bits(b.r);
+        const float X1 = fmaf(ra, a.cs, X), Z1 = fmaf(ra, a.sn, Z);
+        const float d1 = fminf(M.fhw - abs_bits(X1), M.fhh - abs_bits(Z1));
+        const float p1 = dmin * d1;
+        const float X2 = fmaf(rb, b.cs, X1), Z2 = fmaf(rb, b.sn, Z1);
+        const float d2 = fminf(M.fhw - abs_bits(X2), M.fhh - abs_bits(Z2));
+        const float p2 = d1 * d2;
+        if (fminf(p1, p2) <= A.f_bthr) {
+            float U;
+            if (p1 <= A.f_bthr && reaches_wall(M, A, X, Z, X1, Z1, d1, p1, w.x, w.y, U)) {
+                put_exit(X, Z, X1, Z1, U, n + k);
+                return true;
+            }
+            if (p2 <= A.f_bthr && reaches_wall(M, A, X1, Z1, X2, Z2, d2, p2, w.z, w.w, U)) {
+                put_exit(X1, Z1, X2, Z2, U, n + k + 1u);
+                count_step(M, X1, Z1);
                 return true;
             }
         }
-        if constexpr (kRegions) count_regions(M, Xn, Zn);
-        else occ.add(material(M, Xn, Zn));
-        X = Xn;
-        Z = Zn;
-        dmin = dn;
+        count_step(M, X1, Z1);
+        count_step(M, X2, Z2);
+        X = X2;
+        Z = Z2;
+        dmin = d2;
         return false;
-    }
-
-    __device__ __forceinline__ bool substep(const ModelDev &M, const WalkArgs &A, uint32_t wa,
-                                            uint32_t wb, uint32_t k, ExitInfo<float> &ei) {
-        return advance(M, A, increment(A, wa, wb), wa, wb, k, ei);
     }
 
     // Raster programs with up to 8 materials: the walk does not depend on the
@@ -400,7 +454,7 @@ struct WalkerF32 {
 
     // The step of advance() with the material lookup deferred.
     __device__ __forceinline__ bool advance_cell(const ModelDev &M, const WalkArgs &A, const Incr &d,
-                                                 uint32_t wa, uint32_t wb, uint32_t k, ExitInfo<float> &ei,
+                                                 uint32_t wa, uint32_t wb, uint32_t k,
                                                  uint32_t &ci, uint32_t &off) {
         const float nr = neg_bits(d.r);
         const float Xn = fmaf(nr, d.cs, X);
@@ -408,8 +462,9 @@ struct WalkerF32 {
         const float dn = fminf(M.fhw - abs_bits(Xn), M.fhh - abs_bits(Zn));
         const float pn = dmin * dn;
         if (pn <= A.f_bthr) {
-            if (near_wall(M, A, Xn, Zn, dn, pn, wa, wb, ei)) {
-                ei.nocc = n + k;
+            float U;
+            if (reaches_wall(M, A, X, Z, Xn, Zn, dn, pn, wa, wb, U)) {
+                put_exit(X, Z, Xn, Zn, U, n + k);
                 return true;
             }
         }
@@ -451,8 +506,7 @@ struct WalkerF32 {
     // at the end of an iteration).
     static constexpr int PAIRS = KMAX == 8 ? 2 : 4;
 
-    __device__ __forceinline__ int iterate(const ModelDev &M, const WalkArgs &A, uint32_t path,
-                                           ExitInfo<float> &ei) {
+    __device__ __forceinline__ int iterate(const ModelDev &M, const WalkArgs &A, uint32_t, ExitInfo<float> &) {
         uint4 w[PAIRS];
 #pragma unroll
         for (int q = 0; q < PAIRS; ++q) w[q] = philox_rk_pre((n >> 1) + q, 0u, pre_x, pre_y, A.rk0, A.rk1);
@@ -465,7 +519,7 @@ struct WalkerF32 {
                 if (done == NS) {
                     const uint32_t wa = (k & 1) ? w[k >> 1].z : w[k >> 1].x;
                     const uint32_t wb = (k & 1) ? w[k >> 1].w : w[k >> 1].y;
-                    if (advance_cell(M, A, increment(A, wa, wb), wa, wb, (uint32_t)k, ei, ci[k], off[k >> 2]))
+                    if (advance_cell(M, A, increment(A, wa, wb), wa, wb, (uint32_t)k, ci[k], off[k >> 2]))
                         done = k;
                 }
             }
@@ -474,61 +528,146 @@ struct WalkerF32 {
         } else {
 #pragma unroll
             for (int q = 0; q < PAIRS; ++q) {
-                if (substep(M, A, w[q].x, w[q].y, 2u * q, ei)) return 1;
-                if (substep(M, A, w[q].z, w[q].w, 2u * q + 1u, ei)) return 1;
+                if (advance2(M, A, w[q], 2u * q)) return 1;
             }
         }
         n += 2 * PAIRS;
         if (n >= A.max_steps) {
-            ei.x = X; ei.z = Z; ei.th = 0.f; ei.wall = 0;
-            ei.mlast = material(M, X, Z);
-            ei.nocc = n;
+            put_exit(X, Z, X, Z, 0.f, n);
             return 2;
         }
         return 0;
     }
 
-    // Cooperative tail (scheduler): once few walks are left, every lane of
-    // the warp computes increments for them, and each walk then runs only
-    // the position-dependent chain of its steps.  The increments are the
-    // ones increment() gives in iterate(), so the walks are the same.
+    // Cooperative rounds (scheduler): the lanes of a segment of the warp share
+    // one walk.  Lane q of the segment forms the increments of pair q of the
+    // round (two steps), the ones increment() gives in iterate(); every lane
+    // then runs the moves of the pairs before its own, one fused multiply-add
+    // a step and coordinate, and tests its own two steps.  The walk is the
+    // one iterate() makes, bit for bit.
     static constexpr bool kCoop = true;
-    __device__ __forceinline__ uint32_t steps() const { return n; }
-    __device__ __forceinline__ uint2 key() const { return make_uint2(pre_x, pre_y); }
+    using CoopInc = float4;
+    struct Coop {
+        float X, Z;            // the walk's position at the start of the round
+        uint32_t n, kx, ky;    // its step counter and keys
+        uint32_t owner;        // the lane that holds the walk
+        const uint32_t *tco;
+        decltype(WalkerF32::occ) occ;  // this lane's share of the occupation
+        float X0, Z0, X1, Z1, X2, Z2, U;  // before, between and after the lane's two steps
+    };
 
-    // The two increments of Philox pair q of a walk with step counter n0
-    // (even) and key (pre_x, pre_y); the fourth word keeps the high 9 bits of
-    // wa (bits 31..23) and of wb (bits 22..14).
-    __device__ __forceinline__ static void pair_increments(const WalkArgs &A, uint32_t n0, uint2 key,
-                                                           uint32_t q, float4 &s0, float4 &s1) {
-        const uint4 w = philox_rk_pre((n0 >> 1) + q, 0u, key.x, key.y, A.rk0, A.rk1);
-        const Incr a = increment(A, w.x, w.y), b = increment(A, w.z, w.w);
-        s0 = make_float4(a.r, a.sn, a.cs, __uint_as_float((w.x & 0xff800000u) | (w.y >> 9)));
-        s1 = make_float4(b.r, b.sn, b.cs, __uint_as_float((w.z & 0xff800000u) | (w.w >> 9)));
+    __device__ __forceinline__ void coop_begin(Coop &c, int owner, int lane) const {
+        c.X = __shfl_sync(kFull, X, owner);
+        c.Z = __shfl_sync(kFull, Z, owner);
+        c.n = __shfl_sync(kFull, n, owner);
+        c.kx = __shfl_sync(kFull, pre_x, owner);
+        c.ky = __shfl_sync(kFull, pre_y, owner);
+        c.owner = (uint32_t)owner;
+        if (GC == GC_RASTER_MULTI)
+            c.tco = reinterpret_cast<const uint32_t *>(
+                __shfl_sync(kFull, reinterpret_cast<unsigned long long>(tco), owner));
+        if constexpr (KMAX == 8 && !kRegions) c.occ.base = occ.base + 4u * (uint32_t)(owner - lane);
+        else c.occ.clear();
     }
 
-    // Steps with the cnt (even) increments d[0 .. cnt-1].  0 running,
-    // 1 exited, 2 truncated (at max_steps exactly, as in iterate()).
-    __device__ __forceinline__ int consume(const ModelDev &M, const WalkArgs &A, const float4 *d,
-                                           int cnt, ExitInfo<float> &ei) {
-        for (int k = 0; k < cnt; ++k) {
-            const float4 v = d[k];
-            Incr c;
-            c.r = v.x;
-            c.sn = v.y;
-            c.cs = v.z;
-            const uint32_t hb = __float_as_uint(v.w);
-            if (advance(M, A, c, hb & 0xff800000u, hb << 9, (uint32_t)k, ei)) return 1;
-            if (n + (uint32_t)k + 1u >= A.max_steps) {
-                n += (uint32_t)k + 1u;
-                ei.x = X; ei.z = Z; ei.th = 0.f; ei.wall = 0;
-                ei.mlast = material(M, X, Z);
-                ei.nocc = n;
-                return 2;
+    // One round of per pairs.  in: this lane takes part (q < per); buf: the
+    // segment's increments.  0, or this lane's first event: 1 and 2, the first
+    // and the second of its steps ends the walk; 3, max_steps is reached after
+    // both.
+    __device__ __forceinline__ static int coop_round(const ModelDev &M, const WalkArgs &A, Coop &c, CoopInc *buf,
+                                                     uint32_t q, int per, bool in) {
+        const uint4 w = philox_rk_pre((c.n >> 1) + q, 0u, c.kx, c.ky, A.rk0, A.rk1);
+        const Incr a = increment(A, w.x, w.y), b = increment(A, w.z, w.w);
+        const float ra = neg_bits(a.r), rb = neg_bits(b.r);
+        if (in) {
+            buf[2 * q] = make_float4(ra, a.sn, a.cs, 0.f);
+            buf[2 * q + 1] = make_float4(rb, b.sn, b.cs, 0.f);
+        }
+        __syncwarp();
+        float X = c.X, Z = c.Z;
+#pragma unroll 4
+        for (int p = 0; p < per - 1; ++p) {
+            const float4 u = buf[2 * p], v = buf[2 * p + 1];
+            if (p < (int)q) {
+                X = fmaf(u.x, u.z, X);
+                Z = fmaf(u.x, u.y, Z);
+                X = fmaf(v.x, v.z, X);
+                Z = fmaf(v.x, v.y, Z);
             }
         }
-        n += (uint32_t)cnt;
-        return 0;
+        c.X0 = X;
+        c.Z0 = Z;
+        c.X1 = fmaf(ra, a.cs, X);
+        c.Z1 = fmaf(ra, a.sn, Z);
+        c.X2 = fmaf(rb, b.cs, c.X1);
+        c.Z2 = fmaf(rb, b.sn, c.Z1);
+        const float d0 = fminf(M.fhw - abs_bits(c.X0), M.fhh - abs_bits(c.Z0));
+        const float d1 = fminf(M.fhw - abs_bits(c.X1), M.fhh - abs_bits(c.Z1));
+        const float d2 = fminf(M.fhw - abs_bits(c.X2), M.fhh - abs_bits(c.Z2));
+        const float p1 = d0 * d1, p2 = d1 * d2;
+        const uint32_t k = c.n + 2u * q;
+        if (!in || k >= A.max_steps) return 0;
+        if (p1 <= A.f_bthr && reaches_wall(M, A, c.X0, c.Z0, c.X1, c.Z1, d1, p1, w.x, w.y, c.U)) return 1;
+        if (p2 <= A.f_bthr && reaches_wall(M, A, c.X1, c.Z1, c.X2, c.Z2, d2, p2, w.z, w.w, c.U)) return 2;
+        return k + 2u >= A.max_steps ? 3 : 0;
+    }
+
+    // The occupation of this lane's first cnt (0 .. 2) steps of the round.
+    __device__ __forceinline__ static void coop_count(const ModelDev &M, Coop &c, int cnt) {
+        WalkerF32 t;
+        t.occ = c.occ;
+        t.tco = c.tco;
+        if (cnt > 0) t.count_step(M, c.X1, c.Z1);
+        if (cnt > 1) t.count_step(M, c.X2, c.Z2);
+        c.occ = t.occ;
+    }
+
+    // No walk ended in the round: on to the next one (last: the lane of the
+    // segment's last pair).
+    __device__ __forceinline__ static void coop_next(Coop &c, int per, int last) {
+        c.X = __shfl_sync(kFull, c.X2, last);
+        c.Z = __shfl_sync(kFull, c.Z2, last);
+        c.n += 2u * (uint32_t)per;
+    }
+
+    // The lane whose step ended the walk leaves it in the owner's column.
+    __device__ __forceinline__ void coop_put(const Coop &c, int code, uint32_t q, int lane) const {
+        WalkerF32 t;
+        t.pend = pend + 4u * (c.owner - (uint32_t)lane);
+        const uint32_t k = c.n + 2u * q;
+        if (code == 1) t.put_exit(c.X0, c.Z0, c.X1, c.Z1, c.U, k);
+        if (code == 2) t.put_exit(c.X1, c.Z1, c.X2, c.Z2, c.U, k + 1u);
+        if (code == 3) t.put_exit(c.X2, c.Z2, c.X2, c.Z2, 0.f, k + 2u);
+    }
+
+    // The owner takes its walk back: base is the first lane of the walk's
+    // segment (seg: this lane's own segment), last the lane of its last pair.
+    __device__ __forceinline__ void coop_end(const Coop &c, unsigned seg, int per, int base, bool mine) {
+        const float x = __shfl_sync(kFull, c.X2, base + per - 1), z = __shfl_sync(kFull, c.Z2, base + per - 1);
+        const uint32_t m = __shfl_sync(kFull, c.n, base) + 2u * (uint32_t)per;
+        if (mine) {
+            X = x;
+            Z = z;
+            n = m;
+        }
+        if constexpr (kRegions) {
+            const uint32_t e = seg_sum(c.occ.ce, seg), s = seg_sum(c.occ.cs, seg);
+            const uint32_t ge = __shfl_sync(kFull, e, base), gs = __shfl_sync(kFull, s, base);
+            if (mine) {
+                occ.ce += ge;
+                occ.cs += gs;
+            }
+        } else if constexpr (KMAX < 8) {
+#pragma unroll
+            for (int j = 0; j < KMAX - 1; ++j) {
+                const uint32_t e = seg_sum(c.occ.s[j], seg);
+                const uint32_t g = __shfl_sync(kFull, e, base);
+                if (mine) occ.s[j] += g;
+            }
+        }
+    }
+    __device__ __forceinline__ static uint32_t seg_sum(uint32_t v, unsigned seg) {
+        return seg ? __reduce_add_sync(seg, v) : 0u;
     }
 
     __device__ static void to_abs(const ModelDev &M, float X, float Z, double &x, double &z) {

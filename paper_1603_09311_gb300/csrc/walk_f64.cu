@@ -26,6 +26,7 @@ struct WalkerF64 {
     using Real = double;
     static constexpr int KMAX = KMAX_;
     static constexpr bool kCoop = false;  // no cooperative tail: the parity walk stays plain
+    using CoopInc = char;
     static constexpr bool kGrouped = false;  // one queue (a grouped plan's order is one queue too)
     static constexpr int kMinCTAs = 3;
     using Occ = uint32_t;
@@ -70,7 +71,7 @@ struct WalkerF64 {
         }
     }
 
-    __device__ __forceinline__ void bind(HistT *) {}
+    __device__ __forceinline__ void bind(HistT *, float *) {}
 
     __device__ __forceinline__ void counts(const ModelDev &, uint32_t, uint32_t *c) const {
 #pragma unroll
@@ -171,6 +172,10 @@ struct WalkerF64 {
         if (r) return r;
         return substep(M, A, path, w.z, w.w, ei);
     }
+
+    // the step that ends a walk writes its exit record itself
+    static constexpr int kPend = 0;
+    __device__ __forceinline__ void finalize(const ModelDev &, const WalkArgs &, int, ExitInfo<double> &) const {}
 
     __device__ static void to_abs(const ModelDev &, double X, double Z, double &ox, double &oz) {
         ox = X;

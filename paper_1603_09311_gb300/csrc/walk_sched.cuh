@@ -163,13 +163,9 @@ struct WarpSmem {
     Ring<W> ring;
     WarpState st;
     typename W::HistT hist[W::kHist][32];     // per-lane occupation histogram
-    float4 tail[W::kCoop ? 64 : 1];           // step increments of the cooperative tail
+    float pend[W::kPend > 0 ? W::kPend : 1][32];  // exiting steps that wait for their records
+    typename W::CoopInc coop[W::kCoop ? 64 : 1];  // step increments of the cooperative rounds
 };
-
-// A warp whose queue is drained switches to the cooperative tail once it
-// has at most this many walks left.
-constexpr int kTailWalks = 8;
-
 
 template <class W>
 __host__ __device__ constexpr size_t shared_bytes(int warps, int E, int K) {
@@ -191,9 +187,12 @@ struct ExitInfo {
 //   start(M, A, x0, z0, path, node_id, model)  -- begin a walk
 //   iterate(M, A, path, ExitInfo&) -> 0 running, 1 exited, 2 truncated
 //     (a few Euler steps per call; max_steps is a multiple of them)
+//   finalize(M, A, st, ExitInfo&): the exit record of a walk that has ended
 //   counts(M, nocc, c): steps spent in materials 1..KMAX-1 (at the exit,
 //     after nocc occupation steps)
-//   bind(a): shared-memory address of the lane's occupancy histogram
+//   bind(h, p): the lane's columns of the occupancy histogram and of the
+//     exiting steps that wait for their records (kPend words)
+//   kCoop, CoopInc, Coop, coop_*: cooperative rounds
 //   static sample(M, T, A, model, e, x, z, th, wall, mlast, counts) -> double2
 //   static to_abs(M, x, z, ax, az)
 //   kGrouped: takes items from per-model queues (multi-model launches)
@@ -239,7 +238,7 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
 
     // per-lane walk state
     W w;
-    w.bind(&WS.hist[0][lane]);
+    w.bind(&WS.hist[0][lane], &WS.pend[0][lane]);
     bool active = false;
     int item = 0;
     int model = 0;
@@ -332,7 +331,7 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
     // Hand paths to idle lanes, opening the next queued item whenever the
     // current one is fully handed out.
     auto refill = [&]() {
-        unsigned need = __ballot_sync(kFull, !active);
+        unsigned need = __ballot_sync(kFull, !active && lane < A.max_lanes);
         if (A.cancel && need) {
             // a cancelled request: no more paths; the walks in flight end
             int c = 0;
@@ -416,15 +415,15 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
         }
     };
 
-    // Records of the walks that ended this iteration (st: 1 exited,
-    // 2 truncated), then a batch of samples once 32 records are waiting.
+    // Records of the walks that have ended (st: 1 exited, 2 truncated), then
+    // a batch of samples once 32 records are waiting.
     ExitInfo<Real> ei{};
     auto on_exits = [&](int st) {
         const unsigned em = __ballot_sync(kFull, st != 0);
         const int nex = __popc(em);
-        if (st != 0) active = false;
         const uint32_t tail = S.tail;
         if (st != 0) {
+            w.finalize(M, A, st, ei);
             const int slot = (tail + __popc(em & lt_mask)) & (kRing - 1);
             const bool tr = st == 2;
             R.x[slot] = ei.x;
@@ -454,44 +453,77 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
     };
 
     refill();
-    int n_active = __popc(__ballot_sync(kFull, active));
-    while (n_active > 0) {
-        if (W::kCoop && n_active <= kTailWalks && S.queue_empty && S.disp_rem == 0) break;
-        int st = 0;
-        if (active) st = w.iterate(M, A, path, ei);
-        if (__ballot_sync(kFull, st != 0) == 0) continue;
-        on_exits(st);
+    int n_live = __popc(__ballot_sync(kFull, active));  // lanes with a walk, ended ones included
+    // A lane whose walk has ended waits (ended != 0) until exit_batch lanes of
+    // the warp have, or all of them: the records and the refill cost a warp
+    // the same for one ended walk as for several.
+    int ended = 0;
+    int n_batch = min(n_live, A.exit_batch);
+    while (n_live > 0) {
+        if (W::kCoop && n_live <= kCoopWalks &&
+            (A.max_lanes <= kCoopWalks || (S.queue_empty && S.disp_rem == 0)))
+            break;
+        int st = active ? 0 : -1;
+        do {
+            if (st == 0) st = w.iterate(M, A, path, ei);
+        } while (__popc(__ballot_sync(kFull, st > 0)) < n_batch);
+        ended = max(st, 0);
+        active = st == 0;
+        on_exits(ended);
+        ended = 0;
         refill();
-        n_active = __popc(__ballot_sync(kFull, active));
+        n_live = __popc(__ballot_sync(kFull, active));
+        n_batch = min(n_live, A.exit_batch);
     }
 
-    // Cooperative tail: nothing is left to hand out and at most kTailWalks
-    // walks remain.  Each round, lane l computes Philox pair l / a of the
-    // (l mod a)-th live walk (a walks live), so every walk gets 32 / a pairs
-    // of step increments at once; then each live lane runs its 2 (32 / a)
-    // steps from shared memory, whose serial part is only the move, the wall
-    // tests and the material lookup.
+    // Cooperative rounds: the warp has a <= kCoopWalks walks.  Alone in its
+    // lane a walk is one dependent chain of about 250 cycles a step (the
+    // random words, the normals, the move, the tests).  Here each walk gets
+    // 32 / a lanes, two steps a lane and round: the words, the normals and the
+    // tests of all its steps are formed side by side, and only the moves
+    // remain one after the other.  The lanes work for the same walks until
+    // one of them ends.
     if constexpr (W::kCoop) {
-        float4 *buf = WS.tail;
-        while (n_active > 0) {
+        while (n_live > 0) {
             const unsigned act = __ballot_sync(kFull, active);
-            const int a = __popc(act);
-            const int per = 32 / a;
-            const int j = lane % a, q = lane / a;
+            const int per = 32 / n_live;
+            const int j = lane / per;
+            const uint32_t q = (uint32_t)(lane % per);
+            const bool in = j < n_live;
             unsigned m = act;
-            for (int t = 0; t < j; ++t) m &= m - 1u;
-            const int src = __ffs(m) - 1;
-            const uint32_t n0 = __shfl_sync(kFull, w.steps(), src);
-            const uint2 k0 = w.key();
-            const uint2 key = make_uint2(__shfl_sync(kFull, k0.x, src), __shfl_sync(kFull, k0.y, src));
-            if (q < per) W::pair_increments(A, n0, key, (uint32_t)q, buf[j * 2 * per + 2 * q],
-                                            buf[j * 2 * per + 2 * q + 1]);
+            for (int t = 0; t < j && in; ++t) m &= m - 1u;
+            const int owner = __ffs(m) - 1;
+            const unsigned seg = in ? (kFull >> (32 - per)) << (j * per) : 0u;
+            const int last = in ? j * per + per - 1 : lane;
+            typename W::CoopInc *buf = WS.coop + (in ? j * 2 * per : 0);
+            typename W::Coop c;
+            w.coop_begin(c, owner, lane);
+            int code;
+            unsigned events;
+            for (;;) {
+                code = W::coop_round(M, A, c, buf, q, per, in);
+                events = __ballot_sync(kFull, code != 0);
+                if (events) break;
+                W::coop_count(M, c, in ? 2 : 0);
+                W::coop_next(c, per, last);
+                __syncwarp();
+            }
+            // the steps before the segment's first event count (of the event's
+            // lane: those before it)
+            const int first = (events & seg) ? __ffs(events & seg) - 1 : 32;
+            W::coop_count(M, c, !in || lane > first ? 0 : (lane < first ? 2 : (code == 3 ? 2 : code - 1)));
+            if (lane == first) w.coop_put(c, code, q, lane);
+            const int fcode = __shfl_sync(kFull, code, first & 31);
+            const int my_st = first == 32 ? 0 : (fcode == 3 ? 2 : 1);
+            const int base = __popc(act & lt_mask) * per;  // this lane's walk, if it owns one
+            const int st_own = __shfl_sync(kFull, my_st, base & 31);
+            w.coop_end(c, seg, per, active ? base : 0, active);
+            ended = active ? st_own : 0;
+            if (ended) active = false;
             __syncwarp();
-            int st = 0;
-            if (active) st = w.consume(M, A, buf + __popc(act & lt_mask) * 2 * per, 2 * per, ei);
-            __syncwarp();
-            if (__ballot_sync(kFull, st != 0) != 0) on_exits(st);
-            n_active = __popc(__ballot_sync(kFull, active));
+            on_exits(ended);
+            refill();
+            n_live = __popc(__ballot_sync(kFull, active));
         }
     }
     if (S.tail != S.head) process((int)(S.tail - S.head));

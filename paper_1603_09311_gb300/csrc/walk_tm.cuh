@@ -42,6 +42,7 @@ struct WalkerTM {
     static constexpr int KMAX = KMAX_;
     static constexpr bool kF64 = sizeof(Real) == 8;
     static constexpr bool kCoop = false;
+    using CoopInc = char;
     static constexpr bool kGrouped = false;
     static constexpr int kMinCTAs = 3;
     using Occ = Real;  // occupation time of every strip
@@ -58,7 +59,7 @@ struct WalkerTM {
     bool start_on_if;
     Real *h;           // this lane's occupation times: h[32 m] for strip m
 
-    __device__ __forceinline__ void bind(HistT *p) { h = p; }
+    __device__ __forceinline__ void bind(HistT *p, float *) { h = p; }
 
     __device__ __forceinline__ static Real xif(const ModelDev &M, int k) {
         if constexpr (kF64) return M.xif[k]; else return M.fxif[k];
@@ -298,6 +299,10 @@ struct WalkerTM {
         return 0;
     }
 
+    // the step that ends a walk writes its exit record itself
+    static constexpr int kPend = 0;
+    __device__ __forceinline__ void finalize(const ModelDev &, const WalkArgs &, int, ExitInfo<Real> &) const {}
+
     __device__ static void to_abs(const ModelDev &, Real X, Real Z, double &ox, double &oz) {
         ox = (double)X;
         oz = (double)Z;
@@ -381,6 +386,7 @@ struct WalkerTM32 {
     using Real = float;
     static constexpr int KMAX = KMAX_;
     static constexpr bool kCoop = false;
+    using CoopInc = char;
     static constexpr bool kGrouped = false;
     static constexpr int kMinCTAs = 3;
     using Occ = float;
@@ -403,7 +409,7 @@ struct WalkerTM32 {
     bool start_on_if;
     float *h;
 
-    __device__ __forceinline__ void bind(HistT *p) { h = p; }
+    __device__ __forceinline__ void bind(HistT *p, float *) { h = p; }
 
     __device__ __forceinline__ static int strip(const ModelDev &M, float Xc) {
         int k = 0;
@@ -750,6 +756,10 @@ struct WalkerTM32 {
         }
         return 0;
     }
+
+    // the step that ends a walk writes its exit record itself
+    static constexpr int kPend = 0;
+    __device__ __forceinline__ void finalize(const ModelDev &, const WalkArgs &, int, ExitInfo<float> &) const {}
 
     __device__ static void to_abs(const ModelDev &M, float Xc, float Zc, double &x, double &z) {
         x = (double)Xc + M.xc;
