@@ -499,16 +499,26 @@ struct Launch {
     bool coop;   // the walk has cooperative rounds
 };
 
-// Walks a warp takes at a time.  32, one a lane, unless the call has so few
-// walks that every warp of the grid can take its share of them in cooperative
-// rounds: then that share (and items of that size), so that all warps work.
-// One node x 1000 walks at dt 1e-3 took 0.157 ms with one warp for 32 walks
-// and 0.040 ms with a warp for each; 16000 walks 0.172 and 0.080 ms, 32000
-// 0.175 and 0.115 ms.  Above kCoopWalks a warp fills its lanes.
-int warp_lanes(long long total, const Launch &L) {
+// Size of the items of a call with so few walks that the warps of the grid
+// share them evenly and take them in cooperative rounds, so that all warps
+// work; 0: the general cut.  One node x 1000 walks at dt 1e-3 took 0.157 ms
+// with one warp for 32 walks and 0.040 ms with a warp for each; 16000 walks
+// 0.172 and 0.080 ms, 32000 0.175 and 0.115 ms.  Above kCoopWalks walks a warp
+// fills its lanes.  Double precision takes kCoopLanes64 walks a warp at any
+// size and cuts items of that size up to 64 walks a warp (64000 walks 7.9 ->
+// 6.9 ms, one round of items of 32 leaves a fifth of the warps without one).
+int item_share(long long total, const Launch &L) {
+    if (!L.coop || L.chunk > 0) return 0;
     const long long W = std::max<long long>(1, (long long)L.grid * (L.block / 32));
-    const long long share = (total + W - 1) / W;
-    return L.coop && L.chunk == 0 && share <= kCoopWalks ? (int)std::max<long long>(share, 1) : 32;
+    const long long share = std::max<long long>(1, (total + W - 1) / W);
+    if (L.f64) return share <= 64 ? (int)std::min<long long>(share, kCoopLanes64) : 0;
+    return share <= kCoopWalks ? (int)share : 0;
+}
+
+// Walks a warp takes at a time.
+int warp_lanes(long long total, const Launch &L) {
+    const int share = item_share(total, L);
+    return share > 0 ? share : (L.coop && L.f64 ? kCoopLanes64 : 32);
 }
 
 // Key of a launch shape in the tuning cache file: device, lookup program,
@@ -562,7 +572,7 @@ Launch choose_launch(const sdd_ctx *ctx, const sdd_config *cfg, double dt,
     L.chunk = (cfg && cfg->chunk_paths) ? cfg->chunk_paths : 0;
     L.max_steps = (cfg && cfg->max_steps) ? cfg->max_steps : (int64_t)std::ceil(20.0 / dt);
     if (L.max_steps > kMaxSteps) L.max_steps = kMaxSteps;
-    L.coop = !L.f64 && gcode != GC_TM;
+    L.coop = gcode != GC_TM;
     L.max_steps = (L.max_steps + 7) / 8 * 8;  // single-precision walks advance 8 steps per iteration
     return L;
 }
@@ -647,9 +657,8 @@ Plan plan_work(int32_t n_nodes, const int64_t *begin, const int64_t *count, uint
     P.node_item0.assign((size_t)n_nodes + 1, 0);
     for (int j = 0; j < n_nodes; ++j) P.total_paths += count[j];
     auto first = [&](int j) -> int64_t { return begin ? begin[j] : 0; };
-    const int lanes = warp_lanes(P.total_paths, L);
-    if (L.chunk > 0 || lanes < 32) {
-        const int chunk = L.chunk > 0 ? L.chunk : lanes;
+    const int chunk = L.chunk > 0 ? L.chunk : item_share(P.total_paths, L);
+    if (chunk > 0) {
         for (int j = 0; j < n_nodes; ++j) {
             P.node_item0[j] = (int32_t)P.items.size();
             for (int64_t p = 0; p < count[j]; p += chunk) {
@@ -755,8 +764,7 @@ const Plan &plan_cached(sdd_ctx *ctx, int32_t n_nodes, const int64_t *n_paths, u
     key.paths.assign(n_paths, n_paths + n_nodes);
     long long total = 0;
     for (int j = 0; j < n_nodes; ++j) total += n_paths[j];
-    const int lanes = warp_lanes(total, L);
-    key.chunk = lanes < 32 ? lanes : L.chunk;
+    key.chunk = L.chunk > 0 ? L.chunk : item_share(total, L);
     key.factor = key.chunk > 0 ? 0 : L.factor;
     key.warps = key.chunk > 0 ? 0 : (long long)L.grid * (L.block / 32);
     key.offset = p_offset;
@@ -782,6 +790,16 @@ WalkArgs base_args(sdd_ctx *ctx, const Launch &L, double dt, uint64_t seed) {
     // single-precision bridge uniforms are >= 2^-19, so a hit needs
     // 2 d d' / dt <= -ln U <= 19 ln 2; 1e-3 margin for rounding
     A.f_bthr = (float)(19.0 * std::log(2.0) * dt / 2.0 * 1.001);
+    // double precision: a step whose ends are both further than T from every
+    // wall has 2 d d' / dt > 23 and cannot hit one
+    const double T = std::sqrt(11.5 * dt) * 1.0001;
+    const double edge[4] = {ctx->M.xmin + T, ctx->M.xmax - T, ctx->M.zmin + T, ctx->M.zmax - T};
+    for (int k = 0; k < 4; ++k) {
+        int64_t bits;
+        std::memcpy(&bits, &edge[k], sizeof(bits));
+        const int32_t h = (int32_t)(bits >> 32);
+        A.clear[k] = h ^ ((h >> 31) & 0x7fffffff);
+    }
     A.key0 = (uint32_t)(seed & 0xffffffffu);
     A.key1 = (uint32_t)(seed >> 32);
     for (int r = 0; r < 10; ++r) {

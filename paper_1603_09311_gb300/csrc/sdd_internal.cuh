@@ -27,6 +27,13 @@ constexpr int kRing = 64;  // exit records buffered per warp
 // 0.117, 0.115 ms.
 constexpr int kCoopWalks = 16;
 
+// Double-precision walks are always in cooperative rounds, this many to a
+// warp: a warp instruction takes the FP64 pipe as long for one lane as for 32,
+// and with 4 lanes a walk no lane idles until the queue is empty.  64 nodes x
+// 4000 walks, dt 1e-3: one walk a lane 24.7 ms; 16, 8, 4 walks a warp 21.7,
+// 21.0, 21.7 ms.
+constexpr int kCoopLanes64 = 8;
+
 enum Geo : int { GEO_SHAPES = 0, GEO_RASTER = 1, GEO_TM = 2 };
 
 // Material-lookup programs of the single-precision walk, chosen per model so
@@ -153,6 +160,8 @@ struct WalkArgs {
     float f_cdt;               // -2 ln(2) dt: squared step radius = f_cdt * log2(u0)
     float f_c2dt;              // 2 / dt
     float f_bthr;              // bridge filter: d d' above this cannot hit (single precision)
+    int32_t clear[4];          // double precision: ordered high words of x_min + T, x_max - T, z_min + T,
+                               // z_max - T, T the reach of the bridge test (2 T^2 / dt > 23)
     uint32_t key0, key1;       // Philox key (seed)
     uint32_t rk0[10], rk1[10]; // the key of each Philox round (key bumped by the Weyl constants)
     uint32_t max_steps;

@@ -545,7 +545,7 @@ struct WalkerF32 {
     // then runs the moves of the pairs before its own, one fused multiply-add
     // a step and coordinate, and tests its own two steps.  The walk is the
     // one iterate() makes, bit for bit.
-    static constexpr bool kCoop = true;
+    static constexpr bool kCoop = true, kAlone = true;
     using CoopInc = float4;
     struct Coop {
         float X, Z;            // the walk's position at the start of the round

@@ -12,33 +12,43 @@
 // theta = d / (d - d') (first-exit-time estimate, second case); both inside
 // -> hit iff min_w 2 d_w d'_w / dt <= -ln U (first case with kappa_i = 1);
 // else the step counts for the material of beta'.
+//
+// What bounds it: the FP64 pipe, which takes a warp instruction every 64
+// cycles on a quarter of an SM, however many of its lanes are active.  So the
+// common step has no FP64 operation but the normals, the move and the material
+// test, and a warp with few walks shares them among its lanes (cooperative
+// rounds).
 #include "walk_sched.cuh"
 #include "walk_tm.cuh"
 
 namespace sdd {
 
+// (w + 1/2) 2^-32, the exact value: w and the half as mantissa bits of a double
+// in [1, 2), less one (one FP64 operation; a conversion, a sum and a product
+// are three).
 __device__ __forceinline__ double uni32(uint32_t w) {
-    return ((double)w + 0.5) * (1.0 / 4294967296.0);
+    return __hiloint2double((int)(0x3ff00000u | (w >> 12)), (int)((w << 20) | 0x80000u)) - 1.0;
 }
 
 template <int KMAX_, int GEO>
 struct WalkerF64 {
     using Real = double;
     static constexpr int KMAX = KMAX_;
-    static constexpr bool kCoop = false;  // no cooperative tail: the parity walk stays plain
-    using CoopInc = char;
+    static constexpr bool kCoop = true, kAlone = false;  // every walk in cooperative rounds
     static constexpr bool kGrouped = false;  // one queue (a grouped plan's order is one queue too)
-    static constexpr int kMinCTAs = 3;
+    static constexpr int kMinCTAs = 2;       // the FP64 pipe is busy with 16 warps an SM
     using Occ = uint32_t;
     using HistT = uint32_t;
     static constexpr int kStored = KMAX - 1;
     static constexpr int kHist = 1;
+    static constexpr int kPend = 6;
+    static constexpr int kCnt = KMAX > 1 ? KMAX - 1 : 1;
 
     double x, z;
     uint32_t n;
-    uint32_t cnt[KMAX > 1 ? KMAX - 1 : 1];
-    int mcur;
-    uint32_t nid;
+    uint32_t cnt[kCnt];
+    uint32_t path, nid;
+    double *pend;  // the lane's column of the exiting steps that wait for their records
 
     __device__ static int material(const ModelDev &M, double x, double z) {
         if (GEO == GEO_RASTER) {
@@ -71,26 +81,26 @@ struct WalkerF64 {
         }
     }
 
-    __device__ __forceinline__ void bind(HistT *, float *) {}
+    __device__ __forceinline__ void bind(HistT *, double *p) { pend = p; }
 
     __device__ __forceinline__ void counts(const ModelDev &, uint32_t, uint32_t *c) const {
 #pragma unroll
-        for (int j = 0; j < (KMAX > 1 ? KMAX - 1 : 1); ++j) c[j] = cnt[j];
+        for (int j = 0; j < kCnt; ++j) c[j] = cnt[j];
     }
 
-    __device__ __forceinline__ void count(int m) {
+    __device__ __forceinline__ static void count(uint32_t (&c)[kCnt], int m) {
 #pragma unroll
-        for (int j = 1; j < KMAX; ++j) cnt[j - 1] += (m == j) ? 1u : 0u;
+        for (int j = 1; j < KMAX; ++j) c[j - 1] += (m == j) ? 1u : 0u;
     }
 
-    __device__ __forceinline__ void start(const ModelDev &M, const WalkArgs &A, double x0,
-                                          double z0, uint32_t path, uint32_t node_id, int) {
+    __device__ __forceinline__ void start(const ModelDev &, const WalkArgs &, double x0, double z0, uint32_t path_,
+                                          uint32_t node_id, int) {
         x = x0;
         z = z0;
         n = 0;
 #pragma unroll
-        for (int j = 0; j < (KMAX > 1 ? KMAX - 1 : 1); ++j) cnt[j] = 0;
-        mcur = material(M, x0, z0);
+        for (int j = 0; j < kCnt; ++j) cnt[j] = 0;
+        path = path_;
         nid = node_id;
     }
 
@@ -106,20 +116,78 @@ struct WalkerF64 {
         if (w == 3) ei.z = M.zmax;
     }
 
-    __device__ int substep(const ModelDev &M, const WalkArgs &A, uint32_t path, uint32_t wa,
-                           uint32_t wb, ExitInfo<double> &ei) {
+    // The Euler increment sqrt(dt) W of a step from its Philox words.
+    __device__ __forceinline__ static double2 increment(const WalkArgs &A, uint32_t wa, uint32_t wb) {
         const double u0 = uni32(wa), u1 = uni32(wb);
         const double rho = sqrt(-2.0 * log(u0));
         const double ang = 6.283185307179586 * u1;
-        const double w0 = rho * cos(ang);
-        const double w1 = rho * sin(ang);
-        const double xn = x + A.sdt * w0;
-        const double zn = z + A.sdt * w1;
-        const double d[4] = {x - M.xmin, M.xmax - x, z - M.zmin, M.zmax - z};
+        double sn, cs;
+        sincos(ang, &sn, &cs);
+        return make_double2(A.sdt * (rho * cs), A.sdt * (rho * sn));
+    }
+
+    // Whether x is certainly further than the reach T of the bridge test from
+    // both walls (WalkArgs::clear): the high word of a double, with its sign
+    // folded in, orders like the double, so integer compares of high words
+    // decide, on the safe side.
+    __device__ __forceinline__ static int order_hi(double v) {
+        const int h = __double2hiint(v);
+        return h ^ ((h >> 31) & 0x7fffffff);
+    }
+    __device__ __forceinline__ static bool clear_of_walls(const WalkArgs &A, double x, double z) {
+        const int hx = order_hi(x), hz = order_hi(z);
+        return hx > A.clear[0] && hx < A.clear[1] && hz > A.clear[2] && hz < A.clear[3];
+    }
+
+    // Whether step k, (x0, z0) -> (xn, zn), ends the walk; u: its bridge
+    // uniform, negative on an overshoot.  All walls' products are compared
+    // before the one division: min_w fl(q_w / dt) = fl(min_w q_w / dt).
+    __device__ static bool reaches_wall(const ModelDev &M, const WalkArgs &A, uint32_t path, uint32_t nid, uint32_t k,
+                                        double x0, double z0, double xn, double zn, double &u) {
+        const double d[4] = {x0 - M.xmin, M.xmax - x0, z0 - M.zmin, M.zmax - z0};
         const double dn[4] = {xn - M.xmin, M.xmax - xn, zn - M.zmin, M.zmax - zn};
-        if (dn[0] <= 0.0 || dn[1] <= 0.0 || dn[2] <= 0.0 || dn[3] <= 0.0) {
-            double best = 2.0;
-            int bw = 0;
+        u = -1.0;
+        if (dn[0] <= 0.0 || dn[1] <= 0.0 || dn[2] <= 0.0 || dn[3] <= 0.0) return true;
+        double q = 2.0 * d[0] * dn[0];
+#pragma unroll
+        for (int w = 1; w < 4; ++w) {
+            const double e = 2.0 * d[w] * dn[w];
+            if (e < q) q = e;
+        }
+        // -ln U <= 33 ln 2 < 23 for U >= 2^-33: no uniform can hit above 23
+        if (q > 23.000001 * A.dt) return false;
+        const double best = q / A.dt;
+        if (!(best <= 23.0)) return false;
+        const uint4 b = philox4x32_10(make_uint4(k, path, nid, 1u), A.key0, A.key1);
+        u = uni32(b.x);
+        return best <= -log(u);
+    }
+
+    __device__ __forceinline__ static void put_exit(double *p, double x0, double z0, double xn, double zn, double u,
+                                                    uint32_t k) {
+        p[0] = x0;
+        p[32] = z0;
+        p[64] = xn;
+        p[96] = zn;
+        p[128] = u;
+        p[160] = __hiloint2double(0, (int)k);
+    }
+
+    // The exit record of an ended walk (st: 1 reached the boundary,
+    // 2 truncated), with the expressions of the definitions.
+    __device__ __forceinline__ void finalize(const ModelDev &M, const WalkArgs &A, int st, ExitInfo<double> &ei) const {
+        const double x0 = pend[0], z0 = pend[32], xn = pend[64], zn = pend[96], u = pend[128];
+        ei.nocc = (uint32_t)__double2loint(pend[160]);
+        ei.mlast = material(M, x0, z0);
+        if (st == 2) {
+            ei.x = x0; ei.z = z0; ei.th = 0.0; ei.wall = 0;
+            return;
+        }
+        const double d[4] = {x0 - M.xmin, M.xmax - x0, z0 - M.zmin, M.zmax - z0};
+        const double dn[4] = {xn - M.xmin, M.xmax - xn, zn - M.zmin, M.zmax - zn};
+        double best = 2.0;
+        int bw = 0;
+        if (u < 0.0) {
 #pragma unroll
             for (int w = 0; w < 4; ++w) {
                 if (dn[w] <= 0.0) {
@@ -127,55 +195,120 @@ struct WalkerF64 {
                     if (t < best) { best = t; bw = w; }
                 }
             }
-            place(M, x, z, xn, zn, best, bw, ei);
-            ei.mlast = mcur;
-            ei.nocc = n;
-            return 1;
-        }
-        double best = 2.0 * d[0] * dn[0] / A.dt;
-        int bw = 0;
+        } else {
+            best = 2.0 * d[0] * dn[0] / A.dt;
 #pragma unroll
-        for (int w = 1; w < 4; ++w) {
-            const double e = 2.0 * d[w] * dn[w] / A.dt;
-            if (e < best) { best = e; bw = w; }
+            for (int w = 1; w < 4; ++w) {
+                const double e = 2.0 * d[w] * dn[w] / A.dt;
+                if (e < best) { best = e; bw = w; }
+            }
+            best = best / -log(u);
         }
-        // -ln U <= 33 ln 2 < 23 for U >= 2^-33: no uniform can hit above 23
-        if (best <= 23.0) {
-            const uint4 b = philox4x32_10(make_uint4(n, path, nid, 1u), A.key0, A.key1);
-            const double L = -log(uni32(b.x));
-            if (best <= L) {
-                place(M, x, z, xn, zn, best / L, bw, ei);
-                ei.mlast = mcur;
-                ei.nocc = n;
-                return 1;
+        place(M, x0, z0, xn, zn, best, bw, ei);
+    }
+
+    // Cooperative rounds (scheduler): as in the single-precision walk; the
+    // moves are one addition a step and coordinate, and two steps cost about
+    // 110 FP64 operations a lane.  7 nodes x 2001 walks at dt 1e-3: 21.2 ms
+    // with one walk a lane (280 FP64 operations a step, a warp as long as its
+    // longest walk), 1.8 ms so.
+    using CoopInc = double2;
+    struct Coop {
+        double X, Z;
+        uint32_t n, path, nid, owner;
+        uint32_t cnt[kCnt];
+        double X0, Z0, X1, Z1, X2, Z2, U;
+    };
+
+    __device__ __forceinline__ void coop_begin(Coop &c, int owner, int) const {
+        c.X = __shfl_sync(kFull, x, owner);
+        c.Z = __shfl_sync(kFull, z, owner);
+        c.n = __shfl_sync(kFull, n, owner);
+        c.path = __shfl_sync(kFull, path, owner);
+        c.nid = __shfl_sync(kFull, nid, owner);
+        c.owner = (uint32_t)owner;
+#pragma unroll
+        for (int j = 0; j < kCnt; ++j) c.cnt[j] = 0;
+    }
+
+    __device__ __forceinline__ static int coop_round(const ModelDev &M, const WalkArgs &A, Coop &c, CoopInc *buf,
+                                                     uint32_t q, int per, bool in) {
+        const uint4 w = philox_rk(make_uint4((c.n >> 1) + q, c.path, c.nid, 0u), A.rk0, A.rk1);
+        double2 a, b;
+        // one copy of the normals' code, run twice: it is most of the round
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            const double2 d = increment(A, h ? w.z : w.x, h ? w.w : w.y);
+            if (in) buf[2 * q + h] = d;
+            a = h ? a : d;
+            b = d;
+        }
+        __syncwarp();
+        double X = c.X, Z = c.Z;
+#pragma unroll 4
+        for (int p = 0; p < per - 1; ++p) {
+            const double2 u = buf[2 * p], v = buf[2 * p + 1];
+            if (p < (int)q) {
+                X = X + u.x;
+                Z = Z + u.y;
+                X = X + v.x;
+                Z = Z + v.y;
             }
         }
-        const int m = material(M, xn, zn);
-        count(m);
-        x = xn;
-        z = zn;
-        mcur = m;
-        ++n;
-        if (n >= A.max_steps) {
-            ei.x = x; ei.z = z; ei.th = 0.0; ei.wall = 0;
-            ei.mlast = mcur;
-            ei.nocc = n;
-            return 2;
+        c.X0 = X;
+        c.Z0 = Z;
+        c.X1 = X + a.x;
+        c.Z1 = Z + a.y;
+        c.X2 = c.X1 + b.x;
+        c.Z2 = c.Z1 + b.y;
+        const uint32_t k = c.n + 2u * q;
+        if (!in || k >= A.max_steps) return 0;
+        const bool f0 = clear_of_walls(A, c.X0, c.Z0), f1 = clear_of_walls(A, c.X1, c.Z1);
+        const bool f2 = clear_of_walls(A, c.X2, c.Z2);
+        if (!(f0 && f1 && f2)) {
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h)
+                if (reaches_wall(M, A, c.path, c.nid, k + h, h ? c.X1 : c.X0, h ? c.Z1 : c.Z0, h ? c.X2 : c.X1,
+                                 h ? c.Z2 : c.Z1, c.U))
+                    return 1 + h;
         }
-        return 0;
+        return k + 2u >= A.max_steps ? 3 : 0;
     }
 
-    __device__ __forceinline__ int iterate(const ModelDev &M, const WalkArgs &A, uint32_t path,
-                                           ExitInfo<double> &ei) {
-        const uint4 w = philox4x32_10(make_uint4(n >> 1, path, nid, 0u), A.key0, A.key1);
-        const int r = substep(M, A, path, w.x, w.y, ei);
-        if (r) return r;
-        return substep(M, A, path, w.z, w.w, ei);
+    __device__ __forceinline__ static void coop_count(const ModelDev &M, Coop &c, int k) {
+        if (k > 0) count(c.cnt, material(M, c.X1, c.Z1));
+        if (k > 1) count(c.cnt, material(M, c.X2, c.Z2));
     }
 
-    // the step that ends a walk writes its exit record itself
-    static constexpr int kPend = 0;
-    __device__ __forceinline__ void finalize(const ModelDev &, const WalkArgs &, int, ExitInfo<double> &) const {}
+    __device__ __forceinline__ static void coop_next(Coop &c, int per, int last) {
+        c.X = __shfl_sync(kFull, c.X2, last);
+        c.Z = __shfl_sync(kFull, c.Z2, last);
+        c.n += 2u * (uint32_t)per;
+    }
+
+    __device__ __forceinline__ void coop_put(const Coop &c, int code, uint32_t q, int lane) const {
+        double *p = pend + ((int)c.owner - lane);
+        const uint32_t k = c.n + 2u * q;
+        if (code == 1) put_exit(p, c.X0, c.Z0, c.X1, c.Z1, c.U, k);
+        if (code == 2) put_exit(p, c.X1, c.Z1, c.X2, c.Z2, c.U, k + 1u);
+        if (code == 3) put_exit(p, c.X2, c.Z2, c.X2, c.Z2, 0.0, k + 2u);
+    }
+
+    __device__ __forceinline__ void coop_end(const Coop &c, unsigned seg, int per, int base, bool mine) {
+        const double ex = __shfl_sync(kFull, c.X2, base + per - 1), ez = __shfl_sync(kFull, c.Z2, base + per - 1);
+        const uint32_t m = __shfl_sync(kFull, c.n, base) + 2u * (uint32_t)per;
+        if (mine) {
+            x = ex;
+            z = ez;
+            n = m;
+        }
+#pragma unroll
+        for (int j = 0; j < kCnt; ++j) {
+            const uint32_t v = seg ? __reduce_add_sync(seg, c.cnt[j]) : 0u;
+            const uint32_t g = __shfl_sync(kFull, v, base);
+            if (mine) cnt[j] += g;
+        }
+    }
 
     __device__ static void to_abs(const ModelDev &, double X, double Z, double &ox, double &oz) {
         ox = X;

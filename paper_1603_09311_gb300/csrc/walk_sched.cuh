@@ -163,7 +163,7 @@ struct WarpSmem {
     Ring<W> ring;
     WarpState st;
     typename W::HistT hist[W::kHist][32];     // per-lane occupation histogram
-    float pend[W::kPend > 0 ? W::kPend : 1][32];  // exiting steps that wait for their records
+    typename W::Real pend[W::kPend > 0 ? W::kPend : 1][32];  // exiting steps that wait for their records
     typename W::CoopInc coop[W::kCoop ? 64 : 1];  // step increments of the cooperative rounds
 };
 
@@ -192,7 +192,8 @@ struct ExitInfo {
 //     after nocc occupation steps)
 //   bind(h, p): the lane's columns of the occupancy histogram and of the
 //     exiting steps that wait for their records (kPend words)
-//   kCoop, CoopInc, Coop, coop_*: cooperative rounds
+//   kAlone: has iterate(), one walk a lane; kCoop, CoopInc, Coop, coop_*: has
+//     cooperative rounds
 //   static sample(M, T, A, model, e, x, z, th, wall, mlast, counts) -> double2
 //   static to_abs(M, x, z, ax, az)
 //   kGrouped: takes items from per-model queues (multi-model launches)
@@ -458,22 +459,24 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
     // the warp have, or all of them: the records and the refill cost a warp
     // the same for one ended walk as for several.
     int ended = 0;
-    int n_batch = min(n_live, A.exit_batch);
-    while (n_live > 0) {
-        if (W::kCoop && n_live <= kCoopWalks &&
-            (A.max_lanes <= kCoopWalks || (S.queue_empty && S.disp_rem == 0)))
-            break;
-        int st = active ? 0 : -1;
-        do {
-            if (st == 0) st = w.iterate(M, A, path, ei);
-        } while (__popc(__ballot_sync(kFull, st > 0)) < n_batch);
-        ended = max(st, 0);
-        active = st == 0;
-        on_exits(ended);
-        ended = 0;
-        refill();
-        n_live = __popc(__ballot_sync(kFull, active));
-        n_batch = min(n_live, A.exit_batch);
+    if constexpr (W::kAlone) {
+        int n_batch = min(n_live, A.exit_batch);
+        while (n_live > 0) {
+            if (W::kCoop && n_live <= kCoopWalks &&
+                (A.max_lanes <= kCoopWalks || (S.queue_empty && S.disp_rem == 0)))
+                break;
+            int st = active ? 0 : -1;
+            do {
+                if (st == 0) st = w.iterate(M, A, path, ei);
+            } while (__popc(__ballot_sync(kFull, st > 0)) < n_batch);
+            ended = max(st, 0);
+            active = st == 0;
+            on_exits(ended);
+            ended = 0;
+            refill();
+            n_live = __popc(__ballot_sync(kFull, active));
+            n_batch = min(n_live, A.exit_batch);
+        }
     }
 
     // Cooperative rounds: the warp has a <= kCoopWalks walks.  Alone in its

@@ -41,7 +41,7 @@ struct WalkerTM {
     using Real = Real_;
     static constexpr int KMAX = KMAX_;
     static constexpr bool kF64 = sizeof(Real) == 8;
-    static constexpr bool kCoop = false;
+    static constexpr bool kCoop = false, kAlone = true;
     using CoopInc = char;
     static constexpr bool kGrouped = false;
     static constexpr int kMinCTAs = 3;
@@ -59,7 +59,7 @@ struct WalkerTM {
     bool start_on_if;
     Real *h;           // this lane's occupation times: h[32 m] for strip m
 
-    __device__ __forceinline__ void bind(HistT *p, float *) { h = p; }
+    __device__ __forceinline__ void bind(HistT *p, Real *) { h = p; }
 
     __device__ __forceinline__ static Real xif(const ModelDev &M, int k) {
         if constexpr (kF64) return M.xif[k]; else return M.fxif[k];
@@ -385,7 +385,7 @@ template <int KMAX_>
 struct WalkerTM32 {
     using Real = float;
     static constexpr int KMAX = KMAX_;
-    static constexpr bool kCoop = false;
+    static constexpr bool kCoop = false, kAlone = true;
     using CoopInc = char;
     static constexpr bool kGrouped = false;
     static constexpr int kMinCTAs = 3;
@@ -409,7 +409,7 @@ struct WalkerTM32 {
     bool start_on_if;
     float *h;
 
-    __device__ __forceinline__ void bind(HistT *p, float *) { h = p; }
+    __device__ __forceinline__ void bind(HistT *p, Real *) { h = p; }
 
     __device__ __forceinline__ static int strip(const ModelDev &M, float Xc) {
         int k = 0;
