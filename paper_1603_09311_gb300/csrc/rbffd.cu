@@ -23,12 +23,9 @@
 //   assemble_kernel  one thread per unknown: the row (ELL, n slots, column
 //                    -1 for a Dirichlet neighbour), the diagonal and the
 //                    right-hand side
-//   BiCGStab         five launches per iteration: element-wise updates and
-//                    ELL matrix-vector products, each dot product finished
-//                    by the last block of its launch (block partials summed
-//                    in block order), scalars on the device; batches of 8
-//                    iterations replayed as a CUDA graph, the host reading
-//                    the stop flag after each batch
+//   bicgstab_kernel  all iterations in one cooperative launch (up to 1024 a
+//                    launch): element-wise updates, ELL matrix-vector
+//                    products and dot products between grid barriers
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -174,15 +171,18 @@ __global__ void weights_kernel(const double *p, int n, const int32_t *st, int ns
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double A[kMaxStencil][kMaxStencil + 1];
+    const double self = mq(0.0, eps);
     const double xi = p[2 * i], zi = p[2 * i + 1];
     for (int a = 0; a < ns; ++a) {
         const int ja = st[(size_t)i * ns + a];
         const double xa = p[2 * ja], za = p[2 * ja + 1];
-        for (int b = 0; b < ns; ++b) {
+        // the distance is the same both ways
+        for (int b = 0; b < a; ++b) {
             const int jb = st[(size_t)i * ns + b];
             const double r = hypot(xa - p[2 * jb], za - p[2 * jb + 1]);
-            A[a][b] = mq(r * r, eps);
+            A[a][b] = A[b][a] = mq(r * r, eps);
         }
+        A[a][a] = self;
         const double r = hypot(xa - xi, za - zi);
         const double ph = mq(r * r, eps);
         A[a][ns] = (2.0 * eps * eps + eps * eps * eps * eps * r * r) / (ph * ph * ph);
@@ -291,177 +291,392 @@ __global__ void __launch_bounds__(kDotThreads) dot_partial_kernel(const Z *a, co
     }
 }
 
-// Device-side BiCGStab scalars.  stop: 0 running, 1 converged, 2 breakdown.
-// ticket: the block counter of the launch that is finishing a dot product.
+// Device-side BiCGStab scalars.  stop: 0 running, 1 converged, 2 breakdown,
+// 3 a barrier wait ran out.
 struct Scal {
     Z rho, alpha, omega, beta;
     double rnorm2, bnorm2, tol2;
     int iter, stop;
-    unsigned ticket;
 };
 
-// Block reduction of one or two complex values; thread 0 writes the block's
-// partials, then takes a ticket.  Returns true in every thread of the last
-// block to finish, which then holds all partials (read past L1).
-__device__ bool partial_and_ticket(Z v0, Z v1, bool two, Z *part0, Z *part1, unsigned *ticket) {
-    __shared__ Z s0[kDotThreads], s1[kDotThreads];
-    __shared__ bool last;
-    s0[threadIdx.x] = v0;
-    s1[threadIdx.x] = v1;
+// BiCGStab as one persistent kernel.  Per iteration (dinv = 1 / d)
+//   p = r + beta (p - omega v),  y = p / d                     | barrier
+//   v = K y,  alpha = rho / <r^, v>                            | barrier
+//   s = r - alpha v,  z = s / d                                | barrier
+//   t = K z,  omega = <t, s> / <t, t>  (t = 0: s = 0, omega = 0) | barrier
+//   x += alpha y + omega z,  r = s - omega t,  |r|^2 and the stop test,
+//   rho' = <r^, r>,  beta = (rho' / rho)(alpha / omega)        | barrier
+// The rows are cut into blocks of kDotThreads; a dot product is the pairwise
+// sum of each block's rows (halving), then of the blocks.
+//
+// What bounds it: the FP64 pipe (150 operations a row and iteration, a warp
+// instruction every 64 cycles on a quarter of an SM: 10 us with two warps on
+// each) and five barriers of about 1.2 us with the sums behind three of them.
+// Five launches per iteration, replayed as a graph, took 48 us at 32041 rows:
+// each launch drains the chip and reads its vectors again.  Here a thread
+// keeps its row's vectors in registers and its weights in shared memory; only
+// y and z, which the neighbours read, and the block sums go through L2.  What
+// a barrier's wait can hide is put there (alpha y, p - omega v, x, alpha /
+// omega), and the scalars are formed by one warp, real and imaginary parts in
+// its two halves (by every warp they took 60 of 220 operations).
+//   SPLIT 2 gives a block of rows to two CTAs (the even and the odd rows, so
+//   that the halving sums pair the same rows), one warp on each quarter of an
+//   SM: half the FP64 time where there are at most half as many blocks as SMs.
+//   KEEP false: more blocks than resident CTAs; each CTA takes several blocks
+//   and the vectors stay in global memory.
+struct SolveArgs {
+    const double *ew;
+    const int32_t *ecol, *unk;
+    const double *kappa;
+    const Z *dinv, *rh;
+    Z *r, *p, *v, *x, *y, *z, *s, *t;
+    Z *part;         // [5][blocks * SPLIT]: <r^, v>, <t, s>, <t, t>, <r^, r>, <r, r>
+    Scal *S;
+    unsigned *bar;   // barrier arrivals (zero before the launch)
+    int nu, ns, blocks, max_iter;
+};
+
+constexpr long long kBarrierCycles = 4000000000ll;  // about two seconds
+constexpr unsigned kBarrierFail = 0x80000000u;
+
+// Barrier of all CTAs of the (cooperative) launch, in two halves.  A wait that
+// runs out sets the top bit of the counter; every CTA finds it at this wait or
+// its next one, and leaves.
+__device__ __forceinline__ void grid_arrive(unsigned *bar, unsigned &epoch) {
+    epoch += gridDim.x;
     __syncthreads();
-    for (int off = kDotThreads / 2; off > 0; off >>= 1) {
-        if (threadIdx.x < off) {
-            s0[threadIdx.x] = zadd(s0[threadIdx.x], s0[threadIdx.x + off]);
-            if (two) s1[threadIdx.x] = zadd(s1[threadIdx.x], s1[threadIdx.x + off]);
-        }
-        __syncthreads();
-    }
+    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+}
+__device__ __forceinline__ bool grid_wait(unsigned *bar, unsigned epoch, int *ok) {
     if (threadIdx.x == 0) {
-        part0[blockIdx.x] = s0[0];
-        if (two) part1[blockIdx.x] = s1[0];
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        const long long t0 = clock64();
+        unsigned v;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if ((v & kBarrierFail) || v >= epoch) break;
+            if (clock64() - t0 > kBarrierCycles) v = atomicOr(bar, kBarrierFail) | kBarrierFail;
+        }
+        *ok = (v & kBarrierFail) == 0;
     }
     __syncthreads();
-    return last;
+    return *ok != 0;
 }
 
-// The sum of the partials in block order (the last block only).
-__device__ Z sum_partials(const Z *part, int np) {
-    __shared__ Z s[kDotThreads];
-    Z acc = {0.0, 0.0};
-    for (int i = threadIdx.x; i < np; i += blockDim.x) {
-        const double2 v = __ldcg(reinterpret_cast<const double2 *>(part) + i);
-        acc = zadd(acc, Z{v.x, v.y});
-    }
-    s[threadIdx.x] = acc;
-    __syncthreads();
-    for (int off = kDotThreads / 2; off > 0; off >>= 1) {
-        if (threadIdx.x < off) s[threadIdx.x] = zadd(s[threadIdx.x], s[threadIdx.x + off]);
-        __syncthreads();
-    }
-    const Z out = s[0];
-    __syncthreads();
-    return out;
+// Pairwise sum of n <= 256 complex values by one warp: value i pairs with
+// i + 128, then i + 64, ... i + 1 (missing values are zeros); get(i) fetches
+// value i < n.  Below 32 values the lower half of the warp adds the real parts
+// and the upper half the imaginary ones.  Every lane returns the sum.
+template <class F>
+__device__ __forceinline__ Z halving_sum(int n, F get) {
+    const int lane = threadIdx.x & 31;
+    Z a[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) a[k] = 32 * k + lane < n ? get(32 * k + lane) : Z{0.0, 0.0};
+    if (n > 128)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k] = zadd(a[k], a[k + 4]);
+    if (n > 64)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) a[k] = zadd(a[k], a[k + 2]);
+    if (n > 32) a[0] = zadd(a[0], a[1]);
+    const bool up = lane >= 16;
+    const double give = up ? a[0].re : a[0].im;
+    double v = (up ? a[0].im : a[0].re) + __shfl_xor_sync(0xffffffffu, give, 16);
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return {__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, 16)};
 }
 
-__device__ __forceinline__ Z spmv_row(const double *ew, const int32_t *ecol, int nu, int ns, double kap,
-                                      const Z *x, int r) {
+// a / b and a b by a warp that holds both in every lane: the real part in its
+// lower half, the imaginary part in its upper half; the operations are those
+// of zdiv and zmul.
+__device__ __forceinline__ Z halves(double v) {
+    return {__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, 16)};
+}
+__device__ __forceinline__ Z zdiv_warp(Z a, Z b) {
+    const bool up = (threadIdx.x & 31) >= 16;
+    const double d = b.re * b.re + b.im * b.im;
+    const double m = (up ? a.im : a.re) * b.re, k = (up ? a.re : a.im) * b.im;
+    return halves((m + (up ? -k : k)) / d);
+}
+__device__ __forceinline__ Z zmul_warp(Z a, Z b) {
+    const bool up = (threadIdx.x & 31) >= 16;
+    const double m = a.re * (up ? b.im : b.re), k = a.im * (up ? b.re : b.im);
+    return halves(m + (up ? k : -k));
+}
+
+__device__ __forceinline__ Z ldcg(const Z *p) {
+    const double2 v = __ldcg(reinterpret_cast<const double2 *>(p));
+    return {v.x, v.y};
+}
+__device__ __forceinline__ void stcg(Z *p, Z v) {
+    __stcg(reinterpret_cast<double2 *>(p), make_double2(v.re, v.im));
+}
+
+// The sum over all blocks from their partials: up to 1024 blocks, four to a
+// value of the halving sum.
+template <int SPLIT>
+__device__ __forceinline__ Z block_sums(const Z *part, int blocks) {
+    auto one = [&](int b) {
+        return SPLIT == 1 ? ldcg(part + b) : zadd(ldcg(part + 2 * b), ldcg(part + 2 * b + 1));
+    };
+    return halving_sum(blocks < 256 ? blocks : 256, [&](int i) {
+        Z acc = one(i);
+        for (int b = i + 256; b < blocks; b += 256) acc = zadd(acc, one(b));
+        return acc;
+    });
+}
+
+// One row of K times a vector x that other CTAs write (mine: its entry of this
+// row): the slots, then - i kappa x on the diagonal.  w, c: the row's weights
+// and columns, st apart.  The first slot is the row's own node.
+__device__ __forceinline__ Z row_product(const double *w, const int32_t *c, int st, int ns, double kap, const Z *x,
+                                         int row, Z mine) {
     Z acc = {0.0, 0.0};
-    for (int k = 0; k < ns; ++k) {
-        const int c = ecol[(size_t)k * nu + r];
-        if (c >= 0) {
-            const double wv = ew[(size_t)k * nu + r];
-            acc.re += wv * x[c].re;
-            acc.im += wv * x[c].im;
+    if (c[0] >= 0) {
+        const Z q = c[0] == row ? mine : ldcg(x + c[0]);
+        acc = {w[0] * q.re, w[0] * q.im};
+    }
+#pragma unroll 8
+    for (int k = 1; k < ns; ++k) {
+        const int j = c[k * st];
+        if (j >= 0) {
+            const double wv = w[k * st];
+            const Z q = ldcg(x + j);
+            acc.re += wv * q.re;
+            acc.im += wv * q.im;
         }
     }
-    // - i kappa x = kappa (x.im, -x.re)
-    acc.re += kap * x[r].im;
-    acc.im -= kap * x[r].re;
+    acc.re += kap * mine.im;
+    acc.im -= kap * mine.re;
     return acc;
 }
 
-// One BiCGStab iteration is five launches (grid-stride loops over the rows,
-// the dot products finished by each launch's last block; dinv = 1 / d):
-//   update_p      p = r + beta (p - omega v),  y = p / d
-//   spmv_alpha    v = K y,  alpha = rho / <r^, v>
-//   update_s      s = r - alpha v,  z = s / d
-//   spmv_omega    t = K z,  omega = <t, s> / <t, t>  (t = 0: s = 0, omega = 0)
-//   update_x      x += alpha y + omega z,  r = s - omega t,  |r|^2 and the
-//                 stop test, rho' = <r^, r>,  beta = (rho' / rho)(alpha / omega)
-// Every launch does nothing once stop is set.
-__global__ void __launch_bounds__(kDotThreads) update_p_kernel(int n, const Scal *S, const Z *r, const Z *v,
-                                                               const Z *dinv, Z *p, Z *y) {
-    if (S->stop) return;
-    const Z beta = S->beta, omega = S->omega;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const Z pi = zadd(r[i], zmul(beta, zsub(p[i], zmul(omega, v[i]))));
-        p[i] = pi;
-        y[i] = zmul(pi, dinv[i]);
-    }
-}
+template <int SPLIT, bool KEEP>
+__global__ void __launch_bounds__(kDotThreads / SPLIT, 2) bicgstab_kernel(const SolveArgs A) {
+    constexpr int T = kDotThreads / SPLIT;  // rows of a CTA's block (every SPLIT-th of the block)
+    constexpr int W = T / 32;
+    extern __shared__ __align__(16) unsigned char solve_smem[];
+    const int parts = A.blocks * SPLIT, stride = gridDim.x;
+    const int nb = (parts - (int)blockIdx.x + stride - 1) / stride;    // this CTA's blocks
+    const int nbmax = (parts + stride - 1) / stride;
+    Z(*sum)[T] = reinterpret_cast<Z(*)[T]>(solve_smem);                // [2 nbmax][T]
+    double *sw = reinterpret_cast<double *>(sum + 2 * nbmax);          // KEEP: [ns][T]
+    int32_t *sc = reinterpret_cast<int32_t *>(sw + (KEEP ? A.ns * T : 0));  // KEEP: [ns][T]
+    __shared__ struct {
+        Z alpha, omega, beta, rho, aw;
+        double rnorm2;
+        int stop, bar_ok;
+    } sh;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    auto block_of = [&](int i) { return (int)blockIdx.x + i * stride; };
+    auto row_of = [&](int i) { return (block_of(i) / SPLIT) * kDotThreads + t * SPLIT + block_of(i) % SPLIT; };
+    unsigned epoch = 0;
 
-__global__ void __launch_bounds__(kDotThreads) spmv_alpha_kernel(const double *ew, const int32_t *ecol, int nu,
-                                                                 int ns, const int32_t *unk, const double *kappa,
-                                                                 const Z *y, const Z *rh, Z *v, Z *part,
-                                                                 Scal *S) {
-    if (S->stop) return;
-    Z acc = {0.0, 0.0};
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nu; r += gridDim.x * blockDim.x) {
-        const Z vr = spmv_row(ew, ecol, nu, ns, kappa[unk[r]], y, r);
-        v[r] = vr;
-        acc = zadd(acc, zcdot(rh[r], vr));
+    const Scal S0 = *A.S;
+    if (t == 0) {
+        sh.alpha = S0.alpha;
+        sh.omega = S0.omega;
+        sh.beta = S0.beta;
+        sh.rho = S0.rho;
+        sh.rnorm2 = S0.rnorm2;
+        sh.stop = S0.stop;
     }
-    if (!partial_and_ticket(acc, Z{0.0, 0.0}, false, part, nullptr, &S->ticket)) return;
-    const Z rv = sum_partials(part, gridDim.x);
-    if (threadIdx.x == 0) {
-        S->ticket = 0;
-        if (rv.re == 0.0 && rv.im == 0.0) S->stop = 2;
-        else S->alpha = zdiv(S->rho, rv);
-    }
-}
-
-__global__ void __launch_bounds__(kDotThreads) update_s_kernel(int n, const Scal *S, const Z *r, const Z *v,
-                                                               const Z *dinv, Z *s, Z *z) {
-    if (S->stop) return;
-    const Z alpha = S->alpha;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const Z si = zsub(r[i], zmul(alpha, v[i]));
-        s[i] = si;
-        z[i] = zmul(si, dinv[i]);
-    }
-}
-
-__global__ void __launch_bounds__(kDotThreads) spmv_omega_kernel(const double *ew, const int32_t *ecol, int nu,
-                                                                 int ns, const int32_t *unk, const double *kappa,
-                                                                 const Z *z, const Z *s, Z *t, Z *part0,
-                                                                 Z *part1, Scal *S) {
-    if (S->stop) return;
-    Z ts = {0.0, 0.0}, tt = {0.0, 0.0};
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nu; r += gridDim.x * blockDim.x) {
-        const Z tr = spmv_row(ew, ecol, nu, ns, kappa[unk[r]], z, r);
-        t[r] = tr;
-        ts = zadd(ts, zcdot(tr, s[r]));
-        tt = zadd(tt, zcdot(tr, tr));
-    }
-    if (!partial_and_ticket(ts, tt, true, part0, part1, &S->ticket)) return;
-    const Z sts = sum_partials(part0, gridDim.x);
-    const Z stt = sum_partials(part1, gridDim.x);
-    if (threadIdx.x == 0) {
-        S->ticket = 0;
-        S->omega = stt.re == 0.0 ? Z{0.0, 0.0} : zdiv(sts, stt);
-    }
-}
-
-__global__ void __launch_bounds__(kDotThreads) update_x_kernel(int n, const Z *y, const Z *z, const Z *s,
-                                                               const Z *t, const Z *rh, Z *x, Z *r, Z *part0,
-                                                               Z *part1, Scal *S) {
-    if (S->stop) return;
-    const Z alpha = S->alpha, omega = S->omega;
-    Z rr = {0.0, 0.0}, hr = {0.0, 0.0};
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        x[i] = zadd(x[i], zadd(zmul(alpha, y[i]), zmul(omega, z[i])));
-        const Z ri = zsub(s[i], zmul(omega, t[i]));
-        r[i] = ri;
-        rr = zadd(rr, zcdot(ri, ri));
-        hr = zadd(hr, zcdot(rh[i], ri));
-    }
-    if (!partial_and_ticket(rr, hr, true, part0, part1, &S->ticket)) return;
-    const Z srr = sum_partials(part0, gridDim.x);
-    const Z rho = sum_partials(part1, gridDim.x);
-    if (threadIdx.x == 0) {
-        S->ticket = 0;
-        S->rnorm2 = srr.re;
-        S->iter += 1;
-        if (S->rnorm2 <= S->tol2 * S->bnorm2) {
-            S->stop = 1;
-        } else if ((omega.re == 0.0 && omega.im == 0.0) || (rho.re == 0.0 && rho.im == 0.0)) {
-            S->stop = 2;
-        } else {
-            S->beta = zmul(zdiv(rho, S->rho), zdiv(alpha, omega));
-            S->rho = rho;
+    int iter = S0.iter;
+    const double goal = S0.tol2 * S0.bnorm2;
+    // KEEP: this thread's row; pw = p - omega v, ay = alpha y
+    Z r{}, pw{}, v{}, x{}, rh{}, dinv{}, y{}, z{}, s{}, tt{}, ay{};
+    double kap = 0.0;
+    const int row0 = row_of(0);
+    const bool own = row0 < A.nu;
+    if (KEEP) {
+        for (int k = 0; k < A.ns; ++k) {
+            sw[k * T + t] = own ? A.ew[(size_t)k * A.nu + row0] : 0.0;
+            sc[k * T + t] = own ? A.ecol[(size_t)k * A.nu + row0] : -1;
         }
+        if (own) {
+            r = A.r[row0];
+            pw = A.p[row0];
+            x = A.x[row0];
+            rh = A.rh[row0];
+            dinv = A.dinv[row0];
+            kap = A.kappa[A.unk[row0]];
+        }
+    }
+    // the CTA's partials of one or two dot products (two: values 2 i and
+    // 2 i + 1 of sum for its block i), a warp for each
+    auto put_partials = [&](bool two, int slot) {
+        __syncthreads();
+        const int jobs = two ? 2 * nb : nb;
+        for (int j = warp; j < jobs; j += W) {
+            const int i = two ? j >> 1 : j, w = two ? j & 1 : 0;
+            const Z q = halving_sum(T, [&](int k) { return sum[2 * i + w][k]; });
+            if (lane == 0) stcg(A.part + (size_t)(slot + w) * parts + block_of(i), q);
+        }
+    };
+    __syncthreads();
+
+    bool ok = true;
+    for (int it = 0; it < A.max_iter && !sh.stop; ++it) {
+        const Z beta = sh.beta;
+        for (int i = 0; i < nb; ++i) {
+            const int row = KEEP ? row0 : row_of(i);
+            if (row >= A.nu) continue;
+            if (!KEEP) { r = A.r[row]; pw = A.p[row]; dinv = A.dinv[row]; }
+            pw = zadd(r, zmul(beta, pw));  // p
+            y = zmul(pw, dinv);
+            if (!KEEP) A.p[row] = pw;
+            stcg(A.y + row, y);
+        }
+        grid_arrive(A.bar, epoch);
+        if (!(ok = grid_wait(A.bar, epoch, &sh.bar_ok))) break;
+        for (int i = 0; i < nb; ++i) {
+            const int row = KEEP ? row0 : row_of(i);
+            Z d = {0.0, 0.0};
+            if (row < A.nu) {
+                if (KEEP) v = row_product(sw + t, sc + t, T, A.ns, kap, A.y, row, y);
+                else {
+                    v = row_product(A.ew + row, A.ecol + row, A.nu, A.ns, A.kappa[A.unk[row]], A.y, row,
+                                    ldcg(A.y + row));
+                    A.v[row] = v;
+                    rh = A.rh[row];
+                }
+                d = zcdot(rh, v);
+            }
+            sum[2 * i][t] = d;
+        }
+        put_partials(false, 0);
+        grid_arrive(A.bar, epoch);
+        if (!(ok = grid_wait(A.bar, epoch, &sh.bar_ok))) break;
+        if (warp == 0) {
+            const Z rv = block_sums<SPLIT>(A.part, A.blocks);
+            const Z al = zdiv_warp(sh.rho, rv);
+            if (lane == 0) {
+                if (rv.re == 0.0 && rv.im == 0.0) sh.stop = 2;
+                else sh.alpha = al;
+            }
+        }
+        __syncthreads();
+        if (sh.stop) break;
+        const Z alpha = sh.alpha;
+        for (int i = 0; i < nb; ++i) {
+            const int row = KEEP ? row0 : row_of(i);
+            if (row >= A.nu) continue;
+            if (!KEEP) { r = A.r[row]; v = A.v[row]; dinv = A.dinv[row]; }
+            s = zsub(r, zmul(alpha, v));
+            z = zmul(s, dinv);
+            if (!KEEP) A.s[row] = s;
+            stcg(A.z + row, z);
+        }
+        grid_arrive(A.bar, epoch);
+        if (KEEP) ay = zmul(alpha, y);
+        if (!(ok = grid_wait(A.bar, epoch, &sh.bar_ok))) break;
+        for (int i = 0; i < nb; ++i) {
+            const int row = KEEP ? row0 : row_of(i);
+            Z d = {0.0, 0.0}, e = {0.0, 0.0};
+            if (row < A.nu) {
+                if (KEEP) tt = row_product(sw + t, sc + t, T, A.ns, kap, A.z, row, z);
+                else {
+                    tt = row_product(A.ew + row, A.ecol + row, A.nu, A.ns, A.kappa[A.unk[row]], A.z, row,
+                                     ldcg(A.z + row));
+                    A.t[row] = tt;
+                    s = A.s[row];
+                }
+                d = zcdot(tt, s);
+                e.re = tt.re * tt.re + tt.im * tt.im;  // <t, t> is real
+            }
+            sum[2 * i][t] = d;
+            sum[2 * i + 1][t] = e;
+        }
+        put_partials(true, 1);
+        grid_arrive(A.bar, epoch);
+        if (!(ok = grid_wait(A.bar, epoch, &sh.bar_ok))) break;
+        if (warp < 2) {
+            const Z q = block_sums<SPLIT>(A.part + (size_t)(1 + warp) * parts, A.blocks);
+            if (warp == 1 && lane == 0) sh.aw = q;
+            // warp 0 goes on once warp 1 has <t, t>
+            asm volatile("bar.sync 1, 64;" ::: "memory");
+            if (warp == 0) {
+                const Z stt = sh.aw;
+                const Z om = zdiv_warp(q, stt);
+                if (lane == 0) sh.omega = stt.re == 0.0 ? Z{0.0, 0.0} : om;
+            }
+        }
+        __syncthreads();
+        const Z omega = sh.omega;
+        for (int i = 0; i < nb; ++i) {
+            const int row = KEEP ? row0 : row_of(i);
+            Z d = {0.0, 0.0}, e = {0.0, 0.0};
+            if (row < A.nu) {
+                if (!KEEP) { s = A.s[row]; tt = A.t[row]; rh = A.rh[row]; }
+                r = zsub(s, zmul(omega, tt));
+                if (!KEEP) A.r[row] = r;
+                e.re = r.re * r.re + r.im * r.im;
+                d = zcdot(rh, r);
+            }
+            sum[2 * i][t] = d;
+            sum[2 * i + 1][t] = e;
+        }
+        put_partials(true, 3);
+        grid_arrive(A.bar, epoch);
+        for (int i = 0; i < nb; ++i) {
+            const int row = KEEP ? row0 : row_of(i);
+            if (row >= A.nu) continue;
+            if (!KEEP) {
+                x = A.x[row]; pw = A.p[row]; v = A.v[row];
+                ay = zmul(alpha, ldcg(A.y + row));
+                z = ldcg(A.z + row);
+            }
+            x = zadd(x, zadd(ay, zmul(omega, z)));
+            pw = zsub(pw, zmul(omega, v));
+            if (!KEEP) { A.x[row] = x; A.p[row] = pw; }
+        }
+        if (warp == 2) {
+            const Z aw = zdiv_warp(alpha, omega);
+            if (lane == 0) sh.aw = aw;
+        }
+        if (!(ok = grid_wait(A.bar, epoch, &sh.bar_ok))) break;
+        ++iter;
+        if (warp < 2) {
+            const Z q = block_sums<SPLIT>(A.part + (size_t)(3 + warp) * parts, A.blocks);
+            if (warp == 1) {
+                if (lane == 0) sh.rnorm2 = q.re;
+            } else {
+                const Z be = zmul_warp(zdiv_warp(q, sh.rho), sh.aw);
+                __syncwarp();
+                if (lane == 0) {
+                    sh.beta = be;
+                    sh.rho = q;
+                }
+            }
+        }
+        __syncthreads();
+        const double rn = sh.rnorm2;
+        const Z rho = sh.rho;
+        const int stop = rn <= goal ? 1
+                         : (omega.re == 0.0 && omega.im == 0.0) || (rho.re == 0.0 && rho.im == 0.0) ? 2 : 0;
+        if (stop) {
+            __syncthreads();
+            if (t == 0) sh.stop = stop;
+            break;
+        }
+    }
+    __syncthreads();
+    if (KEEP && own) {
+        A.r[row0] = r;
+        A.p[row0] = pw;
+        A.x[row0] = x;
+    }
+    if (blockIdx.x == 0 && t == 0) {
+        Scal S = S0;
+        S.alpha = sh.alpha;
+        S.omega = sh.omega;
+        S.beta = sh.beta;
+        S.rho = sh.rho;
+        S.rnorm2 = sh.rnorm2;
+        S.iter = iter;
+        S.stop = ok ? sh.stop : 3;
+        *A.S = S;
     }
 }
 
@@ -504,6 +719,43 @@ struct RbScratch {
         return e;
     }
 };
+
+template <int SPLIT, bool KEEP>
+cudaError_t launch_solve(const SolveArgs &A, int n_sm, bool *fits, cudaStream_t st) {
+    constexpr int T = kDotThreads / SPLIT;
+    // KEEP: one block a CTA; else at most eight (1024 blocks, two CTAs on each
+    // of at least 64 SMs)
+    const int parts = A.blocks * SPLIT;
+    const int nb = KEEP ? 1 : (parts + 2 * n_sm - 1) / (2 * n_sm);
+    const size_t smem = (size_t)nb * 2 * T * sizeof(Z) +
+                        (KEEP ? (size_t)A.ns * T * (sizeof(double) + sizeof(int32_t)) : 0);
+    auto k = bicgstab_kernel<SPLIT, KEEP>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int per = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, T, smem);
+    if (e != cudaSuccess) return e;
+    *fits = parts <= per * n_sm;
+    if (KEEP && !*fits) return cudaSuccess;
+    if (!KEEP && (long long)per * n_sm * nb < parts) return cudaErrorLaunchOutOfResources;
+    SolveArgs a = A;
+    void *args[] = {&a};
+    return cudaLaunchCooperativeKernel((const void *)k, dim3(std::min(parts, per * n_sm)), dim3(T), args, smem, st);
+}
+
+// Two CTAs a block of rows while that leaves at most one CTA an SM (FP64 time
+// halves, see bicgstab_kernel); one with the row in registers while all blocks
+// are resident; else several blocks a CTA.
+cudaError_t launch_bicgstab(const SolveArgs &A, cudaStream_t st) {
+    int dev = 0, n_sm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    bool fits = false;
+    if (2 * A.blocks <= n_sm) return launch_solve<2, true>(A, n_sm, &fits, st);
+    e = launch_solve<1, true>(A, n_sm, &fits, st);
+    if (e != cudaSuccess || fits) return e;
+    return launch_solve<1, false>(A, n_sm, &fits, st);
+}
 
 sdd_status check_nodes_eps(const double *nodes_xz, int32_t n, int32_t ns, double eps) {
     if (ns < 2 || ns > kMaxStencil) return rb_arg("n_stencil must be in 2 .. SDD_RBFFD_MAX_STENCIL");
@@ -631,8 +883,9 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
     RbScratch S;
     double *d_p, *d_w, *d_vals, *d_kap, *d_ew, *d_u;
     int32_t *d_st, *d_unk, *d_pos, *d_ecol;
-    Z *d_dinv, *d_b, *x, *rr, *rh, *p, *v, *y, *s, *zz, *t, *part0, *part1;
+    Z *d_dinv, *d_b, *x, *rr, *rh, *p, *v, *y, *s, *zz, *t, *part0, *d_part;
     Scal *d_S;
+    unsigned *d_bar;
     RB_CUDA(S.alloc(&d_p, 2 * (size_t)n));
     RB_CUDA(S.alloc(&d_st, (size_t)n * ns));
     RB_CUDA(S.alloc(&d_w, (size_t)n * ns));
@@ -645,8 +898,9 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
     RB_CUDA(S.alloc(&d_u, 2 * (size_t)n));
     for (Z **q : {&d_dinv, &d_b, &x, &rr, &rh, &p, &v, &y, &s, &zz, &t}) RB_CUDA(S.alloc(q, (size_t)nu));
     RB_CUDA(S.alloc(&part0, (size_t)kDotBlocks));
-    RB_CUDA(S.alloc(&part1, (size_t)kDotBlocks));
+    RB_CUDA(S.alloc(&d_part, 5 * 2 * (size_t)kDotBlocks));
     RB_CUDA(S.alloc(&d_S, 1));
+    RB_CUDA(S.alloc(&d_bar, 1));
     RB_CUDA(cudaStreamCreateWithFlags(&S.st, cudaStreamNonBlocking));
     for (int k = 0; k < 5; ++k) RB_CUDA(cudaEventCreate(&S.ev[k]));
     cudaStream_t st = S.st;
@@ -686,47 +940,23 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
     RB_CUDA(cudaMemcpyAsync(d_S, &h_S, sizeof(Scal), cudaMemcpyHostToDevice, st));
     RB_CUDA(cudaEventRecord(S.ev[3], st));
 
-    // iterations in batches of kPoll, replayed as one CUDA graph; the host
-    // reads the scalars after each batch
-    const int gi = std::min(kDotBlocks, (nu + kDotThreads - 1) / kDotThreads);
-    auto iteration = [&]() {
-        update_p_kernel<<<gi, kDotThreads, 0, st>>>(nu, d_S, rr, v, d_dinv, p, y);
-        spmv_alpha_kernel<<<gi, kDotThreads, 0, st>>>(d_ew, d_ecol, nu, ns, d_unk, d_kap, y, rh, v, part0, d_S);
-        update_s_kernel<<<gi, kDotThreads, 0, st>>>(nu, d_S, rr, v, d_dinv, s, zz);
-        spmv_omega_kernel<<<gi, kDotThreads, 0, st>>>(d_ew, d_ecol, nu, ns, d_unk, d_kap, zz, s, t, part0, part1,
-                                                      d_S);
-        update_x_kernel<<<gi, kDotThreads, 0, st>>>(nu, y, zz, s, t, rh, x, rr, part0, part1, d_S);
-    };
-    const int kPoll = 8;
-    cudaGraphExec_t gexec = nullptr;
-    if (max_iter >= kPoll && !h_S.stop) {
-        cudaGraph_t graph;
-        RB_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        for (int q = 0; q < kPoll; ++q) iteration();
-        RB_CUDA(cudaStreamEndCapture(st, &graph));
-        const cudaError_t e = cudaGraphInstantiate(&gexec, graph, 0);
-        cudaGraphDestroy(graph);
-        RB_CUDA(e);
-    }
-    struct GraphGuard {
-        cudaGraphExec_t g;
-        ~GraphGuard() {
-            if (g) cudaGraphExecDestroy(g);
-        }
-    } gguard{gexec};
-    int it = 0;
-    while (it < max_iter && !h_S.stop) {
-        const int batch = std::min(kPoll, max_iter - it);
-        if (batch == kPoll && gexec) {
-            RB_CUDA(cudaGraphLaunch(gexec, st));
-        } else {
-            for (int q = 0; q < batch; ++q) iteration();
-            RB_CUDA(cudaGetLastError());
-        }
+    // iterations, up to kRun in one cooperative launch
+    SolveArgs sa{};
+    sa.ew = d_ew; sa.ecol = d_ecol; sa.unk = d_unk; sa.kappa = d_kap; sa.dinv = d_dinv; sa.rh = rh;
+    sa.r = rr; sa.p = p; sa.v = v; sa.x = x; sa.y = y; sa.z = zz; sa.s = s; sa.t = t;
+    sa.part = d_part; sa.S = d_S; sa.bar = d_bar;
+    sa.nu = nu; sa.ns = ns;
+    sa.blocks = (nu + kDotThreads - 1) / kDotThreads;
+    const int kRun = 1024;
+    for (int it = 0; it < max_iter && !h_S.stop;) {
+        sa.max_iter = std::min(kRun, max_iter - it);
+        RB_CUDA(cudaMemsetAsync(d_bar, 0, sizeof(unsigned), st));
+        RB_CUDA(launch_bicgstab(sa, st));
         RB_CUDA(cudaMemcpyAsync(&h_S, d_S, sizeof(Scal), cudaMemcpyDeviceToHost, st));
         RB_CUDA(cudaStreamSynchronize(st));
-        it += batch;
+        it += sa.max_iter;
     }
+    if (h_S.stop == 3) return (sdd_status)report_error(SDD_E_CUDA, "a wait between the solver's blocks ran out");
     // the true residual |b - K x| / |b|
     spmv_kernel<<<gb, 128, 0, st>>>(d_ew, d_ecol, nu, ns, d_unk, d_kap, x, t);
     residual_kernel<<<gb, 128, 0, st>>>(t, d_b, nu, s);
