@@ -562,7 +562,11 @@ Launch choose_launch(const sdd_ctx *ctx, const sdd_config *cfg, double dt,
         tune_from_file(const_cast<sdd_ctx *>(ctx), L.kmax, ctx->M.gcode, L.f64, dt);
     const bool tuned = gcode_override < 0 && ctx->tune_block > 0;
     L.block = (cfg && cfg->block_threads) ? cfg->block_threads : (tuned ? ctx->tune_block : 256);
-    L.factor = (cfg && cfg->guided_factor) ? cfg->guided_factor : (tuned ? ctx->tune_k : 2);
+    // 4: where nodes' walks differ in length (TM strips of other diffusion) items
+    // of half a warp's share still leave some warps with the long ones (2401
+    // nodes x 4000 TM walks: factor 1, 2, 4, 8: 61.2, 40.1, 34.9, 35.0 ms); on
+    // the TE lines 2 and 4 differ by less than 1 %
+    L.factor = (cfg && cfg->guided_factor) ? cfg->guided_factor : (tuned ? ctx->tune_k : 4);
     const int gcode = gcode_override >= 0 ? gcode_override : ctx->M.gcode;
     int occ = L.f64 ? occupancy_f64(L.kmax, ctx->geo, L.block, ctx->E, ctx->K)
                     : occupancy_f32(L.kmax, gcode, L.block, ctx->E, std::max(ctx->K, L.kmax));
@@ -572,7 +576,7 @@ Launch choose_launch(const sdd_ctx *ctx, const sdd_config *cfg, double dt,
     L.chunk = (cfg && cfg->chunk_paths) ? cfg->chunk_paths : 0;
     L.max_steps = (cfg && cfg->max_steps) ? cfg->max_steps : (int64_t)std::ceil(20.0 / dt);
     if (L.max_steps > kMaxSteps) L.max_steps = kMaxSteps;
-    L.coop = gcode != GC_TM;
+    L.coop = !(L.f64 && gcode == GC_TM);
     L.max_steps = (L.max_steps + 7) / 8 * 8;  // single-precision walks advance 8 steps per iteration
     return L;
 }

@@ -31,23 +31,6 @@ namespace sdd {
 __device__ __forceinline__ float one_plus(uint32_t w) { return mant_one(w); }
 __device__ __forceinline__ float uni23(uint32_t w) { return one_plus(w) - 0.99999994039535522f; }
 
-// |x| and -x as sign bits alone.  Under -ftz=true fabsf() and unary minus
-// flush denormals, which the compiler forms as an addition of their own; the
-// float operations that take these flush their inputs anyway, so the plain
-// forms give the same results as operand modifiers, without an instruction.
-// There were four such additions a step (of about 62 issue slots): the squared
-// radius, its negated root and the two coordinates of the wall distance.
-__device__ __forceinline__ float abs_bits(float x) {
-    float r;
-    asm("abs.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float neg_bits(float x) {
-    float r;
-    asm("neg.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // Occupation counters.  KMAX = 2: the step count of material 1.  KMAX = 3, 4:
 // power sums s_p = sum over steps of m^p (p = 1 .. KMAX-1), which determine
 // the counts of materials 1 .. KMAX-1 (a Vandermonde system, solved once at
@@ -545,7 +528,7 @@ struct WalkerF32 {
     // then runs the moves of the pairs before its own, one fused multiply-add
     // a step and coordinate, and tests its own two steps.  The walk is the
     // one iterate() makes, bit for bit.
-    static constexpr bool kCoop = true, kAlone = true;
+    static constexpr bool kCoop = true, kAlone = true, kEvents = false;
     using CoopInc = float4;
     struct Coop {
         float X, Z;            // the walk's position at the start of the round
@@ -624,7 +607,7 @@ struct WalkerF32 {
 
     // No walk ended in the round: on to the next one (last: the lane of the
     // segment's last pair).
-    __device__ __forceinline__ static void coop_next(Coop &c, int per, int last) {
+    __device__ __forceinline__ void coop_next(Coop &c, int per, int last) {
         c.X = __shfl_sync(kFull, c.X2, last);
         c.Z = __shfl_sync(kFull, c.Z2, last);
         c.n += 2u * (uint32_t)per;

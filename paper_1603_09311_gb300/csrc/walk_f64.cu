@@ -34,7 +34,7 @@ template <int KMAX_, int GEO>
 struct WalkerF64 {
     using Real = double;
     static constexpr int KMAX = KMAX_;
-    static constexpr bool kCoop = true, kAlone = false;  // every walk in cooperative rounds
+    static constexpr bool kCoop = true, kAlone = false, kEvents = false;  // every walk in cooperative rounds
     static constexpr bool kGrouped = false;  // one queue (a grouped plan's order is one queue too)
     static constexpr int kMinCTAs = 2;       // the FP64 pipe is busy with 16 warps an SM
     using Occ = uint32_t;
@@ -280,7 +280,7 @@ struct WalkerF64 {
         if (k > 1) count(c.cnt, material(M, c.X2, c.Z2));
     }
 
-    __device__ __forceinline__ static void coop_next(Coop &c, int per, int last) {
+    __device__ __forceinline__ void coop_next(Coop &c, int per, int last) {
         c.X = __shfl_sync(kFull, c.X2, last);
         c.Z = __shfl_sync(kFull, c.Z2, last);
         c.n += 2u * (uint32_t)per;

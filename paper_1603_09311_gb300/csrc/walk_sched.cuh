@@ -75,6 +75,23 @@ __device__ __forceinline__ float mant_one(uint32_t w) {
     return __uint_as_float(r);
 }
 
+// |x| and -x as sign bits alone.  Under -ftz=true fabsf() and unary minus
+// flush denormals, which the compiler forms as an addition of their own; the
+// float operations that take these flush their inputs anyway, so the plain
+// forms give the same results as operand modifiers, without an instruction.
+// There were four such additions a step (of about 62 issue slots): the squared
+// radius, its negated root and the two coordinates of the wall distance.
+__device__ __forceinline__ float abs_bits(float x) {
+    float r;
+    asm("abs.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float neg_bits(float x) {
+    float r;
+    asm("neg.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // 32 x 32 -> 64-bit product as one wide multiply.
 __device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t &lo, uint32_t &hi) {
     uint64_t p;
@@ -193,7 +210,7 @@ struct ExitInfo {
 //   bind(h, p): the lane's columns of the occupancy histogram and of the
 //     exiting steps that wait for their records (kPend words)
 //   kAlone: has iterate(), one walk a lane; kCoop, CoopInc, Coop, coop_*: has
-//     cooperative rounds
+//     cooperative rounds (kEvents: a round can end without ending a walk)
 //   static sample(M, T, A, model, e, x, z, th, wall, mlast, counts) -> double2
 //   static to_abs(M, x, z, ax, az)
 //   kGrouped: takes items from per-model queues (multi-model launches)
@@ -508,20 +525,25 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
                 events = __ballot_sync(kFull, code != 0);
                 if (events) break;
                 W::coop_count(M, c, in ? 2 : 0);
-                W::coop_next(c, per, last);
+                w.coop_next(c, per, last);
                 __syncwarp();
             }
             // the steps before the segment's first event count (of the event's
             // lane: those before it)
             const int first = (events & seg) ? __ffs(events & seg) - 1 : 32;
-            W::coop_count(M, c, !in || lane > first ? 0 : (lane < first ? 2 : (code == 3 ? 2 : code - 1)));
-            if (lane == first) w.coop_put(c, code, q, lane);
-            const int fcode = __shfl_sync(kFull, code, first & 31);
-            const int my_st = first == 32 ? 0 : (fcode == 3 ? 2 : 1);
-            const int base = __popc(act & lt_mask) * per;  // this lane's walk, if it owns one
-            const int st_own = __shfl_sync(kFull, my_st, base & 31);
-            w.coop_end(c, seg, per, active ? base : 0, active);
-            ended = active ? st_own : 0;
+            const int base = __popc(act & lt_mask) * per & 31;  // this lane's walk, if it owns one
+            if constexpr (W::kEvents) {
+                ended = w.coop_events(M, A, c, code, first, per, active ? base : 0, active, ei);
+                if (__ballot_sync(kFull, ended != 0) == 0) continue;
+            } else {
+                W::coop_count(M, c, !in || lane > first ? 0 : (lane < first ? 2 : (code == 3 ? 2 : code - 1)));
+                if (lane == first) w.coop_put(c, code, q, lane);
+                const int fcode = __shfl_sync(kFull, code, first & 31);
+                const int my_st = first == 32 ? 0 : (fcode == 3 ? 2 : 1);
+                const int st_own = __shfl_sync(kFull, my_st, base);
+                w.coop_end(c, seg, per, active ? base : 0, active);
+                ended = active ? st_own : 0;
+            }
             if (ended) active = false;
             __syncwarp();
             on_exits(ended);

@@ -41,7 +41,7 @@ struct WalkerTM {
     using Real = Real_;
     static constexpr int KMAX = KMAX_;
     static constexpr bool kF64 = sizeof(Real) == 8;
-    static constexpr bool kCoop = false, kAlone = true;
+    static constexpr bool kCoop = false, kAlone = true, kEvents = false;
     using CoopInc = char;
     static constexpr bool kGrouped = false;
     static constexpr int kMinCTAs = 3;
@@ -385,8 +385,8 @@ template <int KMAX_>
 struct WalkerTM32 {
     using Real = float;
     static constexpr int KMAX = KMAX_;
-    static constexpr bool kCoop = false, kAlone = true;
-    using CoopInc = char;
+    static constexpr bool kCoop = true, kAlone = true, kEvents = true;
+    using CoopInc = float4;
     static constexpr bool kGrouped = false;
     static constexpr int kMinCTAs = 3;
     using Occ = float;
@@ -662,11 +662,11 @@ struct WalkerTM32 {
         float sn, cs;
         // r = sqrt(-2 ln(u0) D_i dt) as sqrt(lc log2(u0)); |.| only guards the
         // last-ulp sign of lg2 near u0 = 1
-        const float r = sqrtf(fabsf(lc * __log2f(uni_m(wa))));
+        const float r = sqrtf(abs_bits(lc * __log2f(uni_m(wa))));
         __sincosf(6.28318530718f * uni_m(wb), &sn, &cs);
         const float Xn = fmaf(r, cs, X);
         const float Zn = fmaf(r, sn, Z);
-        const float dn = fminf(M.fhw - fabsf(Xn), M.fhh - fabsf(Zn));
+        const float dn = fminf(M.fhw - abs_bits(Xn), M.fhh - abs_bits(Zn));
         const float dIn = fminf(Xn - xl, xr - Xn);
         const float pn = dmin * dn, pI = dI * dIn;
         if (pn <= wthr || pI <= wthr || first) {
@@ -735,12 +735,21 @@ struct WalkerTM32 {
             }
             done = stop >= 0 ? (uint32_t)stop + 1u : lim;
         }
-        int st = 0;
         if (stop >= 0) {
-            // back to the position before the recorded step; the steps before
-            // it were spent in the current strip
+            // back to the position before the recorded step
             X = pX;
             Z = pZ;
+        }
+        return resolve(M, A, stop, done, ei);
+    }
+
+    // The end of an iteration: the steps before the recorded one (stop >= 0)
+    // or all done ones were spent in the current strip; then the recorded
+    // step's long path and interface event.
+    __device__ __forceinline__ int resolve(const ModelDev &M, const WalkArgs &A, int stop, uint32_t done,
+                                           ExitInfo<float> &ei) {
+        int st = 0;
+        if (stop >= 0) {
             run += (uint32_t)stop;
             st = rare(M, A, pXn, pZn, pwa, pwb, (uint32_t)stop, ei);
         } else {
@@ -755,6 +764,138 @@ struct WalkerTM32 {
             return 2;
         }
         return 0;
+    }
+
+    // Cooperative rounds (scheduler): the lanes of a segment share one walk
+    // as in the TE walk; a round ends with the first step that needs the long
+    // path, which the walk's owner then takes as at the end of iterate().
+    struct Coop {
+        float X, Z;            // the walk's position at the start of the round
+        uint32_t n, kx, ky;
+        float lc, c2, wthr, xl, xr;  // constants of its strip
+        bool first;            // its next step is a hit at t = 0
+        float sX, sZ, sXn, sZn;  // this lane's recorded step (code 1, 2), or where it got to
+        uint32_t wa, wb;
+    };
+
+    __device__ __forceinline__ void coop_begin(Coop &c, int owner, int) const {
+        c.X = __shfl_sync(kFull, X, owner);
+        c.Z = __shfl_sync(kFull, Z, owner);
+        c.n = __shfl_sync(kFull, n, owner);
+        c.kx = __shfl_sync(kFull, pre_x, owner);
+        c.ky = __shfl_sync(kFull, pre_y, owner);
+        c.lc = __shfl_sync(kFull, lc, owner);
+        c.c2 = __shfl_sync(kFull, c2, owner);
+        c.wthr = __shfl_sync(kFull, wthr, owner);
+        c.xl = __shfl_sync(kFull, xl, owner);
+        c.xr = __shfl_sync(kFull, xr, owner);
+        c.first = __shfl_sync(kFull, (int)(n == 0 && start_on_if), owner) != 0;
+    }
+
+    // Whether a step of the products pn, pI needs the long path (the test of
+    // step()).
+    __device__ __forceinline__ static bool needs_long(const Coop &c, float pn, float pI, uint32_t wa, uint32_t wb) {
+        return (pn <= c.wthr || pI <= c.wthr) && bridge_u(wa, wb) <= __expf(-c.c2 * pn) + __expf(-c.c2 * pI);
+    }
+
+    // One round of per pairs.  0, or this lane's first event: 1 and 2, its
+    // first and its second step needs the long path; 3, max_steps is reached.
+    __device__ __forceinline__ static int coop_round(const ModelDev &M, const WalkArgs &A, Coop &c, CoopInc *buf,
+                                                     uint32_t q, int per, bool in) {
+        const uint32_t odd = c.n & 1u;
+        const uint4 w = philox_rk_pre((c.n >> 1) + q, 0u, c.kx, c.ky, A.rk0, A.rk1);
+        float sa, ca, sb, cb;
+        float ra = sqrtf(abs_bits(c.lc * __log2f(uni_m(w.x))));
+        const float rb = sqrtf(abs_bits(c.lc * __log2f(uni_m(w.z))));
+        __sincosf(6.28318530718f * uni_m(w.y), &sa, &ca);
+        __sincosf(6.28318530718f * uni_m(w.w), &sb, &cb);
+        // an odd counter: the first word pair belongs to the step before
+        const bool skip = q == 0u && odd != 0u;
+        if (skip) ra = 0.f;
+        if (in) {
+            buf[2 * q] = make_float4(ra, sa, ca, 0.f);
+            buf[2 * q + 1] = make_float4(rb, sb, cb, 0.f);
+        }
+        __syncwarp();
+        float X = c.X, Z = c.Z;
+#pragma unroll 4
+        for (int p = 0; p < per - 1; ++p) {
+            const float4 u = buf[2 * p], v = buf[2 * p + 1];
+            if (p < (int)q) {
+                X = fmaf(u.x, u.z, X);
+                Z = fmaf(u.x, u.y, Z);
+                X = fmaf(v.x, v.z, X);
+                Z = fmaf(v.x, v.y, Z);
+            }
+        }
+        const float X1 = fmaf(ra, ca, X), Z1 = fmaf(ra, sa, Z);
+        const float X2 = fmaf(rb, cb, X1), Z2 = fmaf(rb, sb, Z1);
+        const float d0 = fminf(M.fhw - abs_bits(X), M.fhh - abs_bits(Z)), i0 = fminf(X - c.xl, c.xr - X);
+        const float d1 = fminf(M.fhw - abs_bits(X1), M.fhh - abs_bits(Z1)), i1 = fminf(X1 - c.xl, c.xr - X1);
+        const float d2 = fminf(M.fhw - abs_bits(X2), M.fhh - abs_bits(Z2)), i2 = fminf(X2 - c.xl, c.xr - X2);
+        const int lim = (int)(A.max_steps - c.n), k = 2 * (int)q - (int)odd;  // k: the first step's index
+        int code = 0;
+        c.sX = X2;
+        c.sZ = Z2;
+        if (in && k < lim) {
+            if (!skip && ((c.first && q == 0u) || needs_long(c, d0 * d1, i0 * i1, w.x, w.y))) code = 1;
+            else if (k + 1 < lim && needs_long(c, d1 * d2, i1 * i2, w.z, w.w)) code = 2;
+            else if (k + 2 >= lim) code = 3;
+            if (code == 1) { c.sX = X; c.sZ = Z; c.sXn = X1; c.sZn = Z1; c.wa = w.x; c.wb = w.y; }
+            if (code == 2) { c.sX = X1; c.sZ = Z1; c.sXn = X2; c.sZn = Z2; c.wa = w.z; c.wb = w.w; }
+            if (code == 3 && k + 2 > lim) { c.sX = X1; c.sZ = Z1; }
+        }
+        return code;
+    }
+
+    __device__ __forceinline__ static void coop_count(const ModelDev &, Coop &, int) {}
+
+    // No event in the round: on to the next one.
+    __device__ __forceinline__ void coop_next(Coop &c, int per, int last) {
+        c.X = __shfl_sync(kFull, c.sX, last);
+        c.Z = __shfl_sync(kFull, c.sZ, last);
+        c.n += 2u * (uint32_t)per - (c.n & 1u);
+        c.first = false;
+    }
+
+    // The owners take their walks back after a round with events (first: the
+    // lane of this lane's segment with the first one, 32 none; base: the first
+    // lane of the owned walk's segment).  The steps of the rounds before were
+    // spent in the current strip.  0 running, 1 exited, 2 truncated.
+    __device__ __forceinline__ int coop_events(const ModelDev &M, const WalkArgs &A, const Coop &c, int code,
+                                               int first, int per, int base, bool mine, ExitInfo<float> &ei) {
+        const int f = __shfl_sync(kFull, first, base);
+        const int src = f < 32 ? f : base + per - 1;
+        const int fc = __shfl_sync(kFull, code, src);
+        const float x = __shfl_sync(kFull, c.sX, src), z = __shfl_sync(kFull, c.sZ, src);
+        const float xn = __shfl_sync(kFull, c.sXn, src), zn = __shfl_sync(kFull, c.sZn, src);
+        const uint32_t wa = __shfl_sync(kFull, c.wa, src), wb = __shfl_sync(kFull, c.wb, src);
+        const uint32_t m = __shfl_sync(kFull, c.n, base);
+        if (!mine) return 0;
+        run += m - n;
+        n = m;
+        X = x;
+        Z = z;
+        const int odd = (int)(n & 1u);
+        int stop = -1;
+        uint32_t done = 2u * (uint32_t)per - (uint32_t)odd;
+        if (f < 32) {
+            if (fc == 3) {
+                done = A.max_steps - n;
+            } else {
+                stop = 2 * (f - base) + fc - 1 - odd;
+                done = (uint32_t)stop + 1u;
+                pXn = xn;
+                pZn = zn;
+                pwa = wa;
+                pwb = wb;
+            }
+        }
+        if (stop < 0) {
+            dmin = fminf(M.fhw - abs_bits(X), M.fhh - abs_bits(Z));
+            dI = fminf(X - xl, xr - X);
+        }
+        return resolve(M, A, stop, done, ei);
     }
 
     // the step that ends a walk writes its exit record itself

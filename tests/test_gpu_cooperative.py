@@ -110,3 +110,31 @@ def test_small_calls_match_the_oracle(paths, precision):
     assert np.all(np.abs(mean - ref["mean"])[:, 0] <= tol)
     one = npth == 1
     assert np.all(np.isnan(se[one])) and np.all(np.isfinite(se[~one]))
+
+
+TM_MODELS = {
+    "analytic": I.tm_analytic(),
+    "three_strips": I.tm_strips((1.0, 4.0, 0.5), (-0.3, 0.25), [[2.0, 20.0, 7.0]]),
+    "equal_pair": I.tm_strips((2.0, 2.0, 8.0, 1.0), (-0.4, 0.1, 0.6), [[2.0, 1.0, 3.0, 4.0]]),
+    "eight": I.tm_strips([1.0, 2.0, 4.0, 2.0, 1.0, 0.5, 3.0, 1.0], np.linspace(-0.6, 0.6, 7), [np.arange(1.0, 9.0)]),
+}
+
+
+@pytest.mark.parametrize("name", sorted(TM_MODELS))
+@pytest.mark.parametrize("x0,max_steps", [(0.07, 0), (-0.3, 0), (0.0, 0), (0.07, 40), (0.0, 8)])
+def test_few_tm_walks_equal_the_walks_of_a_large_launch(name, x0, max_steps):
+    # x0 = -0.3 and 0 lie on interfaces of some of the models (a hit at t = 0)
+    ctx = sdd.sdd_create(TM_MODELS[name])
+
+    def rec(count, **cfg):
+        return sdd.sdd_walk_occupation(ctx, x0, 0.2, 3, 11, count, 1e-3, 77, max_steps=max_steps, **cfg)
+
+    try:
+        big = rec(BIG, chunk_paths=96)
+        for n in (1, 2, 3, 5, 31, 700):
+            _same(rec(n), big, n)
+        for share in (1, 3, 5, 11, 16, 17):
+            n = min(BIG, share * 152 - 7)
+            _same(rec(n, block_threads=32, ctas_per_sm=1), big, n)
+    finally:
+        ctx.close()
