@@ -1019,6 +1019,7 @@ sdd_status sdd_create(const sdd_model_desc *model, sdd_ctx **out) {
         c->M.tcoarse = (const uint32_t *)c->tiles.p;
         c->M.tpool = (const uint8_t *)c->tiles.p + cb;
         c->M.ntx = tile_cols(model->nx);
+        c->M.tbias = (0x4B400000u >> kTileShift) * (uint32_t)(c->M.ntx + 1);
         c->M.tpool_off = (uint32_t)cb;
     }
     *out = c;

@@ -38,8 +38,8 @@ enum Geo : int { GEO_SHAPES = 0, GEO_RASTER = 1, GEO_TM = 2 };
 
 // Material-lookup programs of the single-precision walk, chosen per model so
 // that the common cases run without loops or branches: the layered
-// background alone, exactly one rectangle, exactly one triangle, up to 4 or
-// up to 16 shapes (unrolled, guarded), or the int8 raster.
+// background alone, exactly one rectangle, exactly one triangle, up to 4
+// shapes (unrolled, guarded), up to 16 (a loop), or the int8 raster.
 // GC_CONTACT is one rectangle [x0, >= x_max) x [0, >= z_max): the earth split
 // by a vertical contact at x0 (the quarter-space model), tested with two
 // compares; it takes the same decisions as GC_RECT1 on every inside point.
@@ -122,6 +122,8 @@ struct ModelDev {
     const uint32_t *tcoarse;  // two-level form of the raster (single-precision walk)
     const uint8_t *tpool;
     int32_t ntx;              // tiles per raster row
+    uint32_t tbias;           // what the rounding constant 1.5 x 2^23 adds to a tile index
+                              // formed from its float bits: (bits >> kTileShift) (ntx + 1)
     uint32_t tpool_off;       // bytes from the coarse table to the pool (same for every model
                               // of a batch: the coarse table rounded up to 256 bytes)
     int32_t nx, nz;

@@ -17,7 +17,7 @@
 // The walk runs in centred coordinates X = x - xc, Z = z - zc, so the
 // distance to the nearer wall of each pair is h - |X|.  Two steps share one
 // Philox call (words 0,1 for the even step, 2,3 for the odd one), and one
-// call of iterate() runs 8 steps (4 with 8 materials).
+// call of iterate() runs 8 steps.
 #include <type_traits>
 
 #include "walk_sched.cuh"
@@ -115,8 +115,8 @@ struct Regions {
     __device__ __forceinline__ void clear() { ce = 0u; cs = 0u; }
 };
 
-// GC: the material-lookup program (GeoCode).  Shape parameters are read
-// with compile-time indices, so every one is an immediate constant operand.
+// GC: the material-lookup program (GeoCode).  Up to four shapes' parameters are
+// read with compile-time indices, so every one is an immediate constant operand.
 template <int KMAX_, int GC>
 struct WalkerF32 {
     using Real = float;
@@ -168,29 +168,48 @@ struct WalkerF32 {
             // map's margin tiles repeat the edge cells, so no clamp is needed.
             // Two-level lookup: the coarse entry (L1-resident) is the material
             // of a uniform tile, else the tile's cells in the pool.
-            const int ix = __float_as_int(fmaf(X, M.fsx, M.fox) + 12582912.0f) - 0x4B400000;
-            const int iz = __float_as_int(fmaf(Z, M.fsz, M.foz) + 12582912.0f) - 0x4B400000;
-            const uint32_t *co = GC == GC_RASTER_MULTI ? tco : M.tcoarse;
-            const uint32_t c = __ldg(co + (iz >> kTileShift) * M.ntx + (ix >> kTileShift));
-            if (c & kTileUniform) return (int)(c & 0xffu);
-            const uint8_t *po = reinterpret_cast<const uint8_t *>(co) + M.tpool_off;
-            return (int)__ldg(po + ((size_t)c << (2 * kTileShift)) + ((iz & (kTile - 1)) << kTileShift) +
-                              (ix & (kTile - 1)));
+            //
+            // The magic number's own bits stay in the indices (its low four
+            // are zero) and leave the tile index as one constant, tbias.  The
+            // second load is predicated, not branched around: a tenth of the
+            // points lie in mixed tiles, so most warps have one, and a branch
+            // was taken on nearly every step.  With this, and the lookups of
+            // two steps side by side, 57 nodes x 2e5 walks at dt 1e-3: K = 3
+            // 14.9 -> 13.9 ms, K = 4 12.8 -> 11.9 ms, K = 5 12.7 -> 9.9 ms (8
+            // materials no longer look an iteration's steps up together after
+            // it); 12 models 4.63 -> 3.84 ms.
+            const uint32_t bx = __float_as_uint(fmaf(X, M.fsx, M.fox) + 12582912.0f);
+            const uint32_t bz = __float_as_uint(fmaf(Z, M.fsz, M.foz) + 12582912.0f);
+            const char *co = reinterpret_cast<const char *>(GC == GC_RASTER_MULTI ? tco : M.tcoarse);
+            const uint32_t tile = (bz >> kTileShift) * (uint32_t)M.ntx + (bx >> kTileShift) - M.tbias;
+            const uint32_t c = __ldg(reinterpret_cast<const uint32_t *>(co) + tile);
+            const uint32_t cell = (c << (2 * kTileShift)) | ((bz & (kTile - 1)) << kTileShift) | (bx & (kTile - 1));
+            uint32_t m = c & 0xffu;
+            asm("{\n\t.reg .pred mixed;\n\tsetp.ge.s32 mixed, %1, 0;\n\t@mixed ld.global.nc.u8 %0, [%2];\n\t}"
+                : "+r"(m) : "r"(c), "l"(co + M.tpool_off + (uint64_t)cell));
+            return (int)m;
         }
         const int m = (Z >= M.fzs) ? M.bg_earth : M.bg_air;
         if (GC == GC_LAYER) return m;
         if (GC == GC_RECT1) return in_rect(M.shapes[0], X, Z) ? M.shapes[0].mat : m;
         if (GC == GC_CONTACT) return (Z >= M.fzs && X >= M.shapes[0].f[0]) ? M.shapes[0].mat : m;
         if (GC == GC_TRI1) return in_tri(M.shapes[0], X, Z) ? M.shapes[0].mat : m;
-        constexpr int NS = GC == GC_SHAPES4 ? 4 : kMaxShapes;
+        // up to 4 shapes unrolled (immediate constants), more in a loop: 16
+        // unrolled tests in each of the iteration's 8 steps overflow the
+        // instruction cache (64 nodes x 5e4 walks through 6 shapes, dt 1e-3:
+        // 90.7 ms with 4 materials and 43.4 with 8, 15.3 and 15.2 in the loop)
         int r = m;
+        auto test = [&](const ShapeDev &S) {
+            const bool in = S.kind == 0 ? in_rect(S, X, Z) : in_tri(S, X, Z);
+            r = in ? S.mat : r;
+        };
+        if (GC == GC_SHAPES4) {
 #pragma unroll
-        for (int s = 0; s < NS; ++s) {
-            if (s < M.n_shapes) {
-                const ShapeDev &S = M.shapes[s];
-                const bool in = S.kind == 0 ? in_rect(S, X, Z) : in_tri(S, X, Z);
-                r = in ? S.mat : r;
-            }
+            for (int s = 0; s < 4; ++s)
+                if (s < M.n_shapes) test(M.shapes[s]);
+        } else {
+#pragma unroll 1
+            for (int s = 0; s < M.n_shapes; ++s) test(M.shapes[s]);
         }
         return r;
     }
@@ -416,70 +435,6 @@ struct WalkerF32 {
         return false;
     }
 
-    // Raster programs with up to 8 materials: the walk does not depend on the
-    // materials it crosses, so an iteration records each accepted step's
-    // tile-map coordinates (the coarse index, and the cell's offset in its
-    // tile, 4 to a word) and looks them up together after its steps, as
-    // independent loads in flight at once instead of one dependent chain per
-    // step (measured: +3 % on one 6-material raster, +7.6 % on a 12-model
-    // batch; with K <= 4 the per-step lookup stays faster, 2.6e11 against
-    // 1.7e11 walk-steps/s).
-    static constexpr bool kDeferLookup = (GC == GC_RASTER || GC == GC_RASTER_MULTI) && KMAX == 8;
-
-    __device__ __forceinline__ static void cell_of(const ModelDev &M, float X, float Z, uint32_t &ci,
-                                                   uint32_t &off, int k) {
-        const int ix = __float_as_int(fmaf(X, M.fsx, M.fox) + 12582912.0f) - 0x4B400000;
-        const int iz = __float_as_int(fmaf(Z, M.fsz, M.foz) + 12582912.0f) - 0x4B400000;
-        ci = (uint32_t)((iz >> kTileShift) * M.ntx + (ix >> kTileShift));
-        const uint32_t o = (uint32_t)(((iz & (kTile - 1)) << kTileShift) | (ix & (kTile - 1)));
-        off = (k & 3) == 0 ? o : off | (o << (8 * (k & 3)));
-    }
-
-    // The step of advance() with the material lookup deferred.
-    __device__ __forceinline__ bool advance_cell(const ModelDev &M, const WalkArgs &A, const Incr &d,
-                                                 uint32_t wa, uint32_t wb, uint32_t k,
-                                                 uint32_t &ci, uint32_t &off) {
-        const float nr = neg_bits(d.r);
-        const float Xn = fmaf(nr, d.cs, X);
-        const float Zn = fmaf(nr, d.sn, Z);
-        const float dn = fminf(M.fhw - abs_bits(Xn), M.fhh - abs_bits(Zn));
-        const float pn = dmin * dn;
-        if (pn <= A.f_bthr) {
-            float U;
-            if (reaches_wall(M, A, X, Z, Xn, Zn, dn, pn, wa, wb, U)) {
-                put_exit(X, Z, Xn, Zn, U, n + k);
-                return true;
-            }
-        }
-        cell_of(M, Xn, Zn, ci, off, (int)k);
-        X = Xn;
-        Z = Zn;
-        dmin = dn;
-        return false;
-    }
-
-    // Count the materials of the first cnt recorded steps: all coarse
-    // entries first, then the cells of mixed tiles.
-    template <int NS>
-    __device__ __forceinline__ void add_cells(const ModelDev &M, const uint32_t (&ci)[NS],
-                                              const uint32_t (&off)[(NS + 3) / 4], int cnt) {
-        const uint32_t *co = GC == GC_RASTER_MULTI ? tco : M.tcoarse;
-        const uint8_t *po = reinterpret_cast<const uint8_t *>(co) + M.tpool_off;
-        uint32_t c[NS];
-#pragma unroll
-        for (int j = 0; j < NS; ++j) c[j] = j < cnt ? __ldg(co + ci[j]) : kTileUniform;
-        int m[NS];
-#pragma unroll
-        for (int j = 0; j < NS; ++j) {
-            const uint32_t o = (off[j >> 2] >> (8 * (j & 3))) & 0xffu;
-            m[j] = (c[j] & kTileUniform) ? (int)(c[j] & 0xffu)
-                                         : (int)__ldg(po + ((size_t)c[j] << (2 * kTileShift)) + o);
-        }
-#pragma unroll
-        for (int j = 0; j < NS; ++j)
-            if (j < cnt) occ.add(m[j]);
-    }
-
     // PAIRS Philox calls, two Euler steps each, per call of iterate: the
     // per-iteration work of the scheduler loop (constants, vote, branch) is
     // shared by 2 PAIRS steps.  The calls depend only on the step counter, so
@@ -487,32 +442,15 @@ struct WalkerF32 {
     // (a walk that exits early discards the rest).  0 running, 1 exited,
     // 2 truncated (max_steps is a multiple of 8, so a walk is only truncated
     // at the end of an iteration).
-    static constexpr int PAIRS = KMAX == 8 ? 2 : 4;
+    static constexpr int PAIRS = 4;
 
     __device__ __forceinline__ int iterate(const ModelDev &M, const WalkArgs &A, uint32_t, ExitInfo<float> &) {
         uint4 w[PAIRS];
 #pragma unroll
         for (int q = 0; q < PAIRS; ++q) w[q] = philox_rk_pre((n >> 1) + q, 0u, pre_x, pre_y, A.rk0, A.rk1);
-        if constexpr (kDeferLookup) {
-            constexpr int NS = 2 * PAIRS;
-            uint32_t ci[NS], off[(NS + 3) / 4];
-            int done = NS;
 #pragma unroll
-            for (int k = 0; k < NS; ++k) {
-                if (done == NS) {
-                    const uint32_t wa = (k & 1) ? w[k >> 1].z : w[k >> 1].x;
-                    const uint32_t wb = (k & 1) ? w[k >> 1].w : w[k >> 1].y;
-                    if (advance_cell(M, A, increment(A, wa, wb), wa, wb, (uint32_t)k, ci[k], off[k >> 2]))
-                        done = k;
-                }
-            }
-            add_cells(M, ci, off, done);
-            if (done < NS) return 1;
-        } else {
-#pragma unroll
-            for (int q = 0; q < PAIRS; ++q) {
-                if (advance2(M, A, w[q], 2u * q)) return 1;
-            }
+        for (int q = 0; q < PAIRS; ++q) {
+            if (advance2(M, A, w[q], 2u * q)) return 1;
         }
         n += 2 * PAIRS;
         if (n >= A.max_steps) {
