@@ -9,16 +9,16 @@
 // estimates are independent, so the standard error carried to s is
 // sqrt(sum_j c_j(s)^2 se_j^2).
 //
-// Kernels (all FP64; the work is small next to the walks that produce the
-// knot values):
-//   arc_kernel            arc length of the polyline, one CTA (chunk sums, a
+// Kernels (all FP64; chains of dependent FP64 operations, about 70 cycles
+// each, are the time, so what can be cut into short ones is):
+//   length_kernel         segment lengths of the polyline
+//   arc_kernel            their prefix sums, one CTA (chunk sums, a
 //                         shared-memory scan, chunk prefixes)
-//   spline_factor_kernel  Thomas forward coefficients of the natural-spline
-//                         equations (one thread; at most 4096 knots)
-//   spline_cols_kernel    G = the spline's second derivatives of every unit
-//                         knot vector, one column per thread
-//   interp_kernel         values and standard errors, one thread per target
-//                         and component
+//   spline_factor_kernel  forward coefficients of the natural-spline
+//                         equations, one thread a row
+//   spline_cols_kernel    the spline's second derivatives of every unit knot
+//                         vector, one thread a column, as far as they matter
+//   linear_kernel, spline_kernel  values and standard errors
 //   scatter_kernel        the knots keep their own estimates
 #include <cmath>
 #include <cstdint>
@@ -36,26 +36,35 @@ namespace {
 
 constexpr int kArcThreads = 1024;
 
-__global__ void __launch_bounds__(kArcThreads) arc_kernel(const double *p, int n, double *s) {
+// s[k + 1] = length of segment k
+__global__ void length_kernel(const double *p, int n, double *s) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n - 1) s[k + 1] = hypot(p[2 * k + 2] - p[2 * k], p[2 * k + 3] - p[2 * k + 1]);
+}
+
+// s[0] = 0, s[k] = sum of the lengths s[1 .. k], in place.  One CTA does only
+// the additions: with the square roots in it (twice) it took 60 us for 1025
+// nodes, the two kernels take 12.
+__global__ void __launch_bounds__(kArcThreads) arc_kernel(int n, double *s) {
     __shared__ double part[kArcThreads];
     const int t = threadIdx.x;
     const int segs = n - 1;
     const int per = (segs + kArcThreads - 1) / kArcThreads;
     const int a = min(t * per, segs), b = min(a + per, segs);
     double acc = 0.0;
-    for (int k = a; k < b; ++k) acc += hypot(p[2 * k + 2] - p[2 * k], p[2 * k + 3] - p[2 * k + 1]);
+    for (int k = a; k < b; ++k) acc += s[k + 1];
     part[t] = acc;
     __syncthreads();
     for (int off = 1; off < kArcThreads; off <<= 1) {
         const double v = t >= off ? part[t - off] : 0.0;
         __syncthreads();
-        part[t] += v;
+        if (t >= off) part[t] += v;
         __syncthreads();
     }
     double run = t > 0 ? part[t - 1] : 0.0;
     if (t == 0) s[0] = 0.0;
     for (int k = a; k < b; ++k) {
-        run += hypot(p[2 * k + 2] - p[2 * k], p[2 * k + 3] - p[2 * k + 1]);
+        run += s[k + 1];
         s[k + 1] = run;
     }
 }
@@ -65,18 +74,26 @@ __global__ void __launch_bounds__(kArcThreads) arc_kernel(const double *p, int n
 //   h_{i-1} M_{i-1} + 2 (h_{i-1} + h_i) M_i + h_i M_{i+1}
 //       = 6 ((v_{i+1} - v_i) / h_i - (v_i - v_{i-1}) / h_{i-1}),
 // M_0 = M_{n-1} = 0.  Thomas forward sweep: den_r = 2 (h_{i-1} + h_i) -
-// h_{i-1} cp_{r-1}, cp_r = h_i / den_r.
-__global__ void spline_factor_kernel(const double *s, int n, double *cp, double *den) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double prev = 0.0;
-    for (int r = 0; r < n - 2; ++r) {
+// h_{i-1} cp_{r-1}, cp_r = h_i / den_r; rden = 1 / den.
+//
+// A row's cp depends on the one before through a factor
+// h_{i-1} h_i / den^2 <= 1/12 (den >= 3/2 h_{i-1} + 2 h_i), so a sweep that
+// starts kWarm rows early from any value in [0, 1/2] has the row's cp to
+// 12^-kWarm < 2^-64: every row is a thread's chain of kWarm divisions, not of
+// all rows before it (257 knots: 190 us -> 15 us).
+constexpr int kWarm = 18;
+__global__ void spline_factor_kernel(const double *s, int n, double *cp, double *rden) {
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= n - 2) return;
+    double prev = 0.0, d = 0.0;
+    for (int r = max(row - kWarm, 0); r <= row; ++r) {
         const int i = r + 1;
         const double hl = s[i] - s[i - 1], hr = s[i + 1] - s[i];
-        const double d = 2.0 * (hl + hr) - (r > 0 ? hl * prev : 0.0);
-        den[r] = d;
+        d = 2.0 * (hl + hr) - (r > 0 ? hl * prev : 0.0);
         prev = hr / d;
-        cp[r] = prev;
     }
+    rden[row] = 1.0 / d;
+    cp[row] = prev;
 }
 
 // Knot spacings must be positive (arc lengths of distinct nodes can still
@@ -86,84 +103,175 @@ __global__ void knots_check_kernel(const double *s, int n, int *err) {
     if (i < n && !(s[i] > s[i - 1])) atomicExch(err, 1);
 }
 
-// Column j of G [n][n]: M(e_j), the second derivatives of the natural spline
-// through the unit vector e_j.  The right-hand side of row r (knot i = r + 1)
-// is non-zero for i in {j - 1, j, j + 1} only.
-__global__ void spline_cols_kernel(const double *s, int n, const double *cp, const double *den,
-                                   double *G) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// Column j of G: M(e_j), the second derivatives of the natural spline through
+// the unit vector e_j, kept by diagonals: G[i][j] at band[i (2 kBand + 1) + j -
+// i + kBand], |i - j| <= kBand, zero where not written.  The right-hand side
+// of row r (knot i = r + 1) is non-zero for i in {j - 1, j, j + 1} only, and
+// the entries fall off on both sides by at least 2/3 a row (0.27 on even
+// knots): a column ends where they are below 2^-100 of its largest, after
+// about 53 rows on even knots, at most after kBand, (2/3)^kBand < 2^-93.
+constexpr int kBand = 160;
+constexpr int kBandRow = 2 * kBand + 1;
+//
+// Every knot has a weight, however small, in every target's sum, so a value or
+// standard error that is not finite makes all of its component's results NaN;
+// the dropped weights must not hide one.  The CTAs past the columns (a warp
+// each, `from` on) look component c of v and of se through: spoil[c] is NaN if
+// it has one, else zero.
+__global__ void __launch_bounds__(32)
+    spline_cols_kernel(const double *s, int n, const double *cp, const double *rden, double *band, int from,
+                       const double *v, const double *se, int V, double *spoil) {
+    if ((int)blockIdx.x >= from) {
+        const int c = (int)blockIdx.x - from;
+        const double *u = c < V ? v + c : se + (c - V);
+        bool bad = false;
+        for (int j = threadIdx.x; j < n; j += 32) bad = bad || !isfinite(u[(size_t)j * V]);
+        const bool any = __any_sync(0xffffffffu, bad);
+        if (threadIdx.x == 0) spoil[c] = any ? nan("") : 0.0;
+        return;
+    }
+    const int j = blockIdx.x * 32 + threadIdx.x;
     if (j >= n) return;
     const int m = n - 2;
-    G[j] = 0.0;
-    G[(size_t)(n - 1) * n + j] = 0.0;
-    double dprev = 0.0;
-    for (int r = 0; r < m; ++r) {
+    auto at = [&](int r) -> double & { return band[(size_t)(r + 1) * kBandRow + (j - r - 1 + kBand)]; };
+    const double tiny = 7.888609052210118e-31;  // 2^-100
+    const int r0 = max(j - 2, 0);               // first row with a right-hand side
+    const int rcap = min(m - 1, j - 1 + kBand);
+    double dprev = 0.0, big = 0.0;
+    int r1 = r0 - 1;
+    for (int r = r0; r <= rcap; ++r) {
         const int i = r + 1;
-        const double hl = s[i] - s[i - 1], hr = s[i + 1] - s[i];
+        const double hl = s[i] - s[i - 1];
         double rhs = 0.0;
-        if (j == i - 1) rhs = 6.0 / hl;
-        else if (j == i) rhs = -(6.0 / hl + 6.0 / hr);
-        else if (j == i + 1) rhs = 6.0 / hr;
-        const double d = (rhs - (r > 0 ? hl * dprev : 0.0)) / den[r];
-        G[(size_t)i * n + j] = d;
+        if (j >= i - 1 && j <= i + 1) {
+            const double hr = s[i + 1] - s[i];
+            if (j == i - 1) rhs = 6.0 / hl;
+            else if (j == i) rhs = -(6.0 / hl + 6.0 / hr);
+            else rhs = 6.0 / hr;
+        }
+        const double d = (rhs - hl * dprev) * rden[r];
+        at(r) = d;
         dprev = d;
+        r1 = r;
+        big = fmax(big, fabs(d));
+        if (r > j && fabs(d) < tiny * big) break;
     }
     double xnext = 0.0;
-    for (int r = m - 1; r >= 0; --r) {
-        const size_t o = (size_t)(r + 1) * n + j;
-        const double x = G[o] - (r < m - 1 ? cp[r] * xnext : 0.0);
-        G[o] = x;
+    const int rend = max(0, j - 1 - kBand);
+    for (int r = r1; r >= rend; --r) {
+        const double x = (r >= r0 ? at(r) : 0.0) - (r < m - 1 ? cp[r] * xnext : 0.0);
+        at(r) = x;
         xnext = x;
+        big = fmax(big, fabs(x));
+        if (r < r0 && fabs(x) < tiny * big) break;
     }
 }
 
-// Thread (target q, component c).  The target's segment is the largest
-// i <= nk - 2 with s_i <= t; with a = (s_{i+1} - t) / h and b = (t - s_i) / h
-//   linear  c_i = a, c_{i+1} = b
-//   spline  c_j = a [j = i] + b [j = i + 1]
-//                 + (a^3 - a) h^2 / 6 G[i][j] + (b^3 - b) h^2 / 6 G[i+1][j]
-// (G == nullptr selects the linear interpolant).
-__global__ void interp_kernel(const double *sk, int nk, const double *G, const double *v,
-                              const double *se, int V, const double *t, int nt, double *ov,
-                              double *ose) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)nt * V) return;
-    const int q = (int)(idx / V), c = (int)(idx % V);
-    const double x = t[q];
+// The target's segment: the largest i <= nk - 2 with s_i <= x.
+__device__ __forceinline__ int segment(const double *sk, int nk, double x) {
     int lo = 0, hi = nk - 2;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (sk[mid] <= x) lo = mid;
         else hi = mid - 1;
     }
-    const int i = lo;
+    return lo;
+}
+
+// Thread (target q, component c): with a = (s_{i+1} - t) / h and
+// b = (t - s_i) / h the weights are c_i = a, c_{i+1} = b.
+__global__ void linear_kernel(const double *sk, int nk, const double *v, const double *se, int V, const double *t,
+                              int nt, double *ov, double *ose) {
+    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (long long)nt * V) return;
+    const int q = (int)(idx / V), c = (int)(idx % V);
+    const double x = t[q];
+    const int i = segment(sk, nk, x);
     const double h = sk[i + 1] - sk[i];
     const double a = (sk[i + 1] - x) / h, b = (x - sk[i]) / h;
-    double val, var = 0.0;
-    if (!G) {
-        const double v0 = v[(size_t)i * V + c], v1 = v[(size_t)(i + 1) * V + c];
-        val = a * v0 + b * v1;
+    const double v0 = v[(size_t)i * V + c], v1 = v[(size_t)(i + 1) * V + c];
+    ov[idx] = a * v0 + b * v1;
+    if (ose) {
+        double var = 0.0;
         if (se) {
             const double e0 = a * se[(size_t)i * V + c], e1 = b * se[(size_t)(i + 1) * V + c];
             var = e0 * e0 + e1 * e1;
         }
-    } else {
-        const double al = (a * a * a - a) * h * h / 6.0, be = (b * b * b - b) * h * h / 6.0;
-        const double *gi = G + (size_t)i * nk, *gi1 = G + (size_t)(i + 1) * nk;
-        val = 0.0;
-        for (int j = 0; j < nk; ++j) {
-            double cj = al * gi[j] + be * gi1[j];
-            if (j == i) cj += a;
-            if (j == i + 1) cj += b;
-            val += cj * v[(size_t)j * V + c];
-            if (se) {
-                const double e = cj * se[(size_t)j * V + c];
+        ose[idx] = sqrt(var);
+    }
+}
+
+// CTA q: target q.  The weights
+//   c_j = a [j = i] + b [j = i + 1]
+//         + (a^3 - a) h^2 / 6 G[i][j] + (b^3 - b) h^2 / 6 G[i+1][j]
+// are formed once, a thread each, then every thread adds up components.  Zero
+// weights (beyond the columns' ends) are skipped.  With a thread for each
+// target and component and all knots in each sum, 1025 targets x 32
+// components x 257 knots took 0.35 ms; 0.05 ms so.
+constexpr int kSplineThreads = 64;
+constexpr int kWeights = 2 * kBand + 2;
+__global__ void __launch_bounds__(kSplineThreads)
+    spline_kernel(const double *sk, int nk, const double *band, const double *v, const double *se, int V,
+                  const double *spoil, const double *t, double *ov, double *ose) {
+    __shared__ double w[kWeights];
+    __shared__ int16_t at[kWeights];
+    __shared__ int count;
+    const size_t q = blockIdx.x;
+    const double x = t[q];
+    const int i = segment(sk, nk, x);
+    const double h = sk[i + 1] - sk[i];
+    const double a = (sk[i + 1] - x) / h, b = (x - sk[i]) / h;
+    const double al = (a * a * a - a) * h * h / 6.0, be = (b * b * b - b) * h * h / 6.0;
+    const int j0 = max(i - kBand, 0), j1 = min(i + 1 + kBand, nk - 1);
+    for (int k = threadIdx.x; k <= j1 - j0; k += kSplineThreads) {
+        const int j = j0 + k, d = j - i;
+        double c = 0.0;
+        if (d <= kBand) c = al * band[(size_t)i * kBandRow + d + kBand];
+        if (d - 1 >= -kBand) c += be * band[(size_t)(i + 1) * kBandRow + d - 1 + kBand];
+        if (d == 0) c += a;
+        if (d == 1) c += b;
+        w[k] = c;
+    }
+    __syncthreads();
+    // the non-zero weights, in order
+    if (threadIdx.x < 32) {
+        int n = 0;
+        for (int k0 = 0; k0 <= j1 - j0; k0 += 32) {
+            const int k = k0 + threadIdx.x;
+            const double c = k <= j1 - j0 ? w[k] : 0.0;
+            const unsigned m = __ballot_sync(0xffffffffu, c != 0.0);
+            __syncwarp();
+            if (c != 0.0) {
+                const int o = n + __popc(m & ((1u << threadIdx.x) - 1u));
+                w[o] = c;
+                at[o] = (int16_t)k;
+            }
+            n += __popc(m);
+            __syncwarp();
+        }
+        if (threadIdx.x == 0) count = n;
+    }
+    __syncthreads();
+    const int n = count;
+    for (int c = threadIdx.x; c < V; c += kSplineThreads) {
+        double val = spoil[c], var = se ? spoil[V + c] : 0.0;
+        const double *vc = v + (size_t)j0 * V + c;
+        if (se) {
+            const double *ec = se + (size_t)j0 * V + c;
+#pragma unroll 4
+            for (int k = 0; k < n; ++k) {
+                const size_t o = (size_t)at[k] * V;
+                val += w[k] * vc[o];
+                const double e = w[k] * ec[o];
                 var += e * e;
             }
+        } else {
+#pragma unroll 4
+            for (int k = 0; k < n; ++k) val += w[k] * vc[(size_t)at[k] * V];
         }
+        ov[q * V + c] = val;
+        if (ose) ose[q * V + c] = sqrt(var);
     }
-    ov[idx] = val;
-    if (ose) ose[idx] = sqrt(var);
 }
 
 __global__ void gather_kernel(const double *s, const int32_t *idx, int nk, double *out) {
@@ -219,23 +327,29 @@ sdd_status run_interp(const double *d_sk, int nk, const double *d_v, const doubl
     INTERP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
     knots_check_kernel<<<(nk + 127) / 128, 128, 0, st>>>(d_sk, nk, err);
     INTERP_CUDA(cudaGetLastError());
-    const double *G = nullptr;
-    if (kind == SDD_INTERP_SPLINE && nk > 2) {
-        double *g, *cp, *den;
-        INTERP_CUDA(S.alloc(&g, (size_t)nk * nk));
-        INTERP_CUDA(S.alloc(&cp, (size_t)nk));
-        INTERP_CUDA(S.alloc(&den, (size_t)nk));
-        spline_factor_kernel<<<1, 32, 0, st>>>(d_sk, nk, cp, den);
-        INTERP_CUDA(cudaGetLastError());
-        spline_cols_kernel<<<(nk + 127) / 128, 128, 0, st>>>(d_sk, nk, cp, den, g);
-        INTERP_CUDA(cudaGetLastError());
-        G = g;
-    }
     const long long total = (long long)nt * V;
-    if (total > 0) {
+    if (kind == SDD_INTERP_SPLINE && nk > 2) {
+        double *band, *cp, *rden, *spoil;
+        const int jobs = d_se ? 2 * V : V, cols = (nk + 31) / 32;
+        const size_t nband = (size_t)nk * kBandRow;
+        INTERP_CUDA(S.alloc(&band, nband));
+        INTERP_CUDA(S.alloc(&cp, (size_t)nk));
+        INTERP_CUDA(S.alloc(&rden, (size_t)nk));
+        INTERP_CUDA(S.alloc(&spoil, (size_t)jobs));
+        INTERP_CUDA(cudaMemsetAsync(band, 0, nband * sizeof(double), st));
+        spline_factor_kernel<<<(nk + 63) / 64, 64, 0, st>>>(d_sk, nk, cp, rden);
+        INTERP_CUDA(cudaGetLastError());
+        spline_cols_kernel<<<cols + jobs, 32, 0, st>>>(d_sk, nk, cp, rden, band, cols, d_v, d_se, V, spoil);
+        INTERP_CUDA(cudaGetLastError());
+        if (total > 0) {
+            spline_kernel<<<(unsigned)nt, kSplineThreads, 0, st>>>(d_sk, nk, band, d_v, d_se, V, spoil, d_t, d_ov,
+                                                                   d_ose);
+            INTERP_CUDA(cudaGetLastError());
+        }
+    } else if (total > 0) {
         const int threads = 128;
-        interp_kernel<<<(unsigned)((total + threads - 1) / threads), threads, 0, st>>>(
-            d_sk, nk, G, d_v, d_se, V, d_t, nt, d_ov, d_ose);
+        linear_kernel<<<(unsigned)((total + threads - 1) / threads), threads, 0, st>>>(d_sk, nk, d_v, d_se, V, d_t, nt,
+                                                                                      d_ov, d_ose);
         INTERP_CUDA(cudaGetLastError());
     }
     INTERP_CUDA(cudaMemcpyAsync(h_err, err, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -373,7 +487,9 @@ extern "C" sdd_status sdd_interface_values_interp(sdd_ctx *ctx, const double *no
     INTERP_CUDA(cudaEventCreate(&ev[1]));
     eg.n = 2;
     INTERP_CUDA(cudaEventRecord(ev[0], st));
-    arc_kernel<<<1, kArcThreads, 0, st>>>(p, n_nodes, s);
+    length_kernel<<<(n_nodes + 127) / 128, 128, 0, st>>>(p, n_nodes, s);
+    INTERP_CUDA(cudaGetLastError());
+    arc_kernel<<<1, kArcThreads, 0, st>>>(n_nodes, s);
     INTERP_CUDA(cudaGetLastError());
     gather_kernel<<<(nk + 127) / 128, 128, 0, st>>>(s, di, nk, sk);
     INTERP_CUDA(cudaGetLastError());
@@ -392,8 +508,8 @@ extern "C" sdd_status sdd_interface_values_interp(sdd_ctx *ctx, const double *no
         float ms = 0.f;
         INTERP_CUDA(cudaEventElapsedTime(&ms, ev[0], ev[1]));
         stats->post_ms = ms;
-        // arc length, knot gather, knot check, [spline factor, spline columns], interpolation, scatter
-        stats->launches += (kind == SDD_INTERP_SPLINE && nk > 2) ? 7 : 5;
+        // lengths, arc length, knot gather, knot check, [spline factor, spline columns], interpolation, scatter
+        stats->launches += (kind == SDD_INTERP_SPLINE && nk > 2) ? 8 : 6;
         stats->h2d_bytes += 2 * (uint64_t)n_nodes * sizeof(double) + (uint64_t)nk * sizeof(int32_t) +
                             2 * (uint64_t)nk * V * sizeof(double);
         stats->d2h_bytes += 2 * (uint64_t)ob * sizeof(double) + sizeof(int);
