@@ -288,17 +288,19 @@ __global__ void scatter_kernel(const double *kv, const double *kse, const int32_
     ose[(size_t)idx[j] * V + c] = kse[e];
 }
 
-// Device allocations of one call, freed on every return path.
+// Stream and device allocations of one call, released on every return path.
 struct Scratch {
     std::vector<void *> ptrs;
+    cudaStream_t st = nullptr;
     ~Scratch() {
-        for (void *p : ptrs) cudaFree(p);
+        for (void *p : ptrs) cudaFreeAsync(p, st);
+        if (st) cudaStreamDestroy(st);
     }
+    cudaError_t open() { return cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking); }
     template <class T>
     cudaError_t alloc(T **p, size_t count) {
         *p = nullptr;
-        if (count == 0) count = 1;
-        cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
+        cudaError_t e = scratch_alloc((void **)p, count * sizeof(T), st);
         if (e == cudaSuccess) ptrs.push_back(*p);
         return e;
     }
@@ -385,6 +387,8 @@ extern "C" sdd_status sdd_interpolate(const double *knots_s, int32_t n_knots, co
     const bool with_se = se != nullptr && out_se != nullptr;
     const size_t kb = (size_t)n_knots * n_vals, tb = (size_t)n_targets * n_vals;
     Scratch S;
+    INTERP_CUDA(S.open());
+    const cudaStream_t st = S.st;
     double *sk, *v, *e = nullptr, *t, *ov, *oe = nullptr;
     INTERP_CUDA(S.alloc(&sk, n_knots));
     INTERP_CUDA(S.alloc(&v, kb));
@@ -394,12 +398,6 @@ extern "C" sdd_status sdd_interpolate(const double *knots_s, int32_t n_knots, co
         INTERP_CUDA(S.alloc(&e, kb));
         INTERP_CUDA(S.alloc(&oe, tb));
     }
-    cudaStream_t st;
-    INTERP_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-    struct StreamGuard {
-        cudaStream_t s;
-        ~StreamGuard() { cudaStreamDestroy(s); }
-    } guard{st};
     INTERP_CUDA(cudaMemcpyAsync(sk, knots_s, n_knots * sizeof(double), cudaMemcpyHostToDevice, st));
     INTERP_CUDA(cudaMemcpyAsync(v, values, kb * sizeof(double), cudaMemcpyHostToDevice, st));
     INTERP_CUDA(cudaMemcpyAsync(t, targets_s, n_targets * sizeof(double), cudaMemcpyHostToDevice, st));
@@ -454,6 +452,8 @@ extern "C" sdd_status sdd_interface_values_interp(sdd_ctx *ctx, const double *no
     if (mc != SDD_OK && mc != SDD_E_TRUNCATED) return mc;
 
     Scratch S;
+    INTERP_CUDA(S.open());
+    const cudaStream_t st = S.st;
     double *p, *s, *sk, *kv, *ke, *ov, *oe;
     int32_t *di;
     const size_t ob = (size_t)n_nodes * V;
@@ -465,12 +465,6 @@ extern "C" sdd_status sdd_interface_values_interp(sdd_ctx *ctx, const double *no
     INTERP_CUDA(S.alloc(&ke, (size_t)nk * V));
     INTERP_CUDA(S.alloc(&ov, ob));
     INTERP_CUDA(S.alloc(&oe, ob));
-    cudaStream_t st;
-    INTERP_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-    struct StreamGuard {
-        cudaStream_t s;
-        ~StreamGuard() { cudaStreamDestroy(s); }
-    } guard{st};
     INTERP_CUDA(cudaMemcpyAsync(p, nodes_xz, 2 * (size_t)n_nodes * sizeof(double), cudaMemcpyHostToDevice, st));
     INTERP_CUDA(cudaMemcpyAsync(di, kidx.data(), nk * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     INTERP_CUDA(cudaMemcpyAsync(kv, kmean.data(), (size_t)nk * V * sizeof(double), cudaMemcpyHostToDevice, st));

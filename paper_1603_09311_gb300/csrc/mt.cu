@@ -108,13 +108,13 @@ struct MtScratch {
     cudaStream_t st = nullptr;
     cudaEvent_t ev[2] = {nullptr, nullptr};
     ~MtScratch() {
-        for (void *p : ptrs) cudaFree(p);
+        for (void *p : ptrs) cudaFreeAsync(p, st);
         for (cudaEvent_t e : ev)
             if (e) cudaEventDestroy(e);
         if (st) cudaStreamDestroy(st);
     }
     cudaError_t alloc(double **p, size_t count) {
-        cudaError_t e = cudaMalloc((void **)p, (count ? count : 1) * sizeof(double));
+        cudaError_t e = scratch_alloc((void **)p, count * sizeof(double), st);
         if (e == cudaSuccess) ptrs.push_back(*p);
         return e;
     }
@@ -130,6 +130,7 @@ sdd_status mt_post(const double *mean, const double *se, int n_sites, int E, dou
     double *dm, *ds, *dk, *dd = nullptr, *orho, *oph, *orse = nullptr, *opse = nullptr, *ou0 = nullptr,
                                                                                        *ouz = nullptr;
     const size_t nv = (size_t)3 * n_sites * E * 2, no = (size_t)n_sites * E;
+    MT_CUDA(cudaStreamCreateWithFlags(&S.st, cudaStreamNonBlocking));
     MT_CUDA(S.alloc(&dm, nv));
     MT_CUDA(S.alloc(&ds, nv));
     MT_CUDA(S.alloc(&dk, E));
@@ -140,7 +141,6 @@ sdd_status mt_post(const double *mean, const double *se, int n_sites, int E, dou
     if (phase_se) MT_CUDA(S.alloc(&opse, no));
     if (u0) MT_CUDA(S.alloc(&ou0, 2 * no));
     if (uz) MT_CUDA(S.alloc(&ouz, 2 * no));
-    MT_CUDA(cudaStreamCreateWithFlags(&S.st, cudaStreamNonBlocking));
     MT_CUDA(cudaEventCreate(&S.ev[0]));
     MT_CUDA(cudaEventCreate(&S.ev[1]));
     cudaStream_t st = S.st;

@@ -706,15 +706,17 @@ struct RbScratch {
     std::vector<void *> ptrs;
     cudaStream_t st = nullptr;
     cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    // a failed call may return with work in flight on st: the releases are
+    // ordered behind it
     ~RbScratch() {
-        for (void *p : ptrs) cudaFree(p);
+        for (void *p : ptrs) cudaFreeAsync(p, st);
         for (cudaEvent_t e : ev)
             if (e) cudaEventDestroy(e);
         if (st) cudaStreamDestroy(st);
     }
     template <class T>
     cudaError_t alloc(T **p, size_t count) {
-        cudaError_t e = cudaMalloc((void **)p, (count ? count : 1) * sizeof(T));
+        cudaError_t e = scratch_alloc((void **)p, count * sizeof(T), st);
         if (e == cudaSuccess) ptrs.push_back(*p);
         return e;
     }
@@ -833,12 +835,12 @@ extern "C" sdd_status sdd_rbffd_weights(const double *nodes_xz, int32_t n, int32
     if (r != SDD_OK) return r;
     if (!stencil || !weights) return rb_arg("stencil and weights must not be NULL");
     RbScratch S;
+    RB_CUDA(cudaStreamCreateWithFlags(&S.st, cudaStreamNonBlocking));
     double *d_p, *d_w;
     int32_t *d_st;
     RB_CUDA(S.alloc(&d_p, 2 * (size_t)n));
     RB_CUDA(S.alloc(&d_st, (size_t)n * n_stencil));
     RB_CUDA(S.alloc(&d_w, (size_t)n * n_stencil));
-    RB_CUDA(cudaStreamCreateWithFlags(&S.st, cudaStreamNonBlocking));
     for (int k = 0; k < 3; ++k) RB_CUDA(cudaEventCreate(&S.ev[k]));
     RB_CUDA(cudaMemcpyAsync(d_p, nodes_xz, 2 * (size_t)n * sizeof(double), cudaMemcpyHostToDevice, S.st));
     r = weights_device(nodes_xz, d_p, n, n_stencil, eps, d_st, d_w, S);
@@ -881,6 +883,7 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
 
     const int ns = n_stencil;
     RbScratch S;
+    RB_CUDA(cudaStreamCreateWithFlags(&S.st, cudaStreamNonBlocking));
     double *d_p, *d_w, *d_vals, *d_kap, *d_ew, *d_u;
     int32_t *d_st, *d_unk, *d_pos, *d_ecol;
     Z *d_dinv, *d_b, *x, *rr, *rh, *p, *v, *y, *s, *zz, *t, *part0, *d_part;
@@ -901,7 +904,6 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
     RB_CUDA(S.alloc(&d_part, 5 * 2 * (size_t)kDotBlocks));
     RB_CUDA(S.alloc(&d_S, 1));
     RB_CUDA(S.alloc(&d_bar, 1));
-    RB_CUDA(cudaStreamCreateWithFlags(&S.st, cudaStreamNonBlocking));
     for (int k = 0; k < 5; ++k) RB_CUDA(cudaEventCreate(&S.ev[k]));
     cudaStream_t st = S.st;
     RB_CUDA(cudaMemcpyAsync(d_p, nodes_xz, 2 * (size_t)n * sizeof(double), cudaMemcpyHostToDevice, st));

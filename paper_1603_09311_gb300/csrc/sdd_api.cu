@@ -941,6 +941,37 @@ sdd_status run(sdd_ctx *ctx, const Plan &P, const Launch &L, WalkArgs A, cudaStr
 
 }  // namespace
 
+cudaError_t sdd::scratch_alloc(void **p, size_t bytes, cudaStream_t st) {
+    static std::mutex mu;
+    static std::map<int, cudaMemPool_t> pools;  // one a device, for the life of the process
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        auto it = pools.find(dev);
+        if (it == pools.end()) {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            e = cudaMemPoolCreate(&pool, &props);
+            if (e != cudaSuccess) return e;
+            uint64_t keep = kScratchKeep;
+            e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) {
+                cudaMemPoolDestroy(pool);
+                return e;
+            }
+            pools[dev] = pool;
+        } else {
+            pool = it->second;
+        }
+    }
+    return cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, st);
+}
+
 int sdd::report_error(int status, const char *msg) { return (int)fail((sdd_status)status, msg); }
 
 int sdd::ctx_site_diffusion(const sdd_ctx *c, double x, double *D) {
