@@ -784,6 +784,25 @@ const Plan &plan_cached(sdd_ctx *ctx, int32_t n_nodes, const int64_t *n_paths, u
     return ctx->plan;
 }
 
+// Whether every phase of the model fits PhaseTurn at this dt.
+bool phases_fit(const ModelDev &M, double dt) {
+    for (int i = 0; i < M.E * M.K; ++i)
+        if (!(M.kappa[i] >= 0.0 && M.kappa[i] * dt * 0.08 < kMaxTurns)) return false;
+    return true;
+}
+
+// The sample constants of a model of a batched launch.
+void fill_samples(BatchModel &B, const ModelDev &M, double dt) {
+    for (int k = 0; k < M.E; ++k) B.ev[k] = eval_f(M.ev[k]);
+    B.turns = phases_fit(M, dt);
+    if (!B.turns) return;
+    for (int k = 0; k < M.E * M.K; ++k) {
+        const PhaseTurn p = phase_turn(M.kappa[k], dt);
+        B.turn_frac[k] = p.frac;
+        B.turn_whole[k] = p.whole;
+    }
+}
+
 WalkArgs base_args(sdd_ctx *ctx, const Launch &L, double dt, uint64_t seed) {
     WalkArgs A;
     std::memset(&A, 0, sizeof(A));
@@ -811,6 +830,7 @@ WalkArgs base_args(sdd_ctx *ctx, const Launch &L, double dt, uint64_t seed) {
         A.rk1[r] = A.key1 + (uint32_t)r * 0xBB67AE85u;
     }
     A.max_steps = (uint32_t)L.max_steps;
+    A.turns = phases_fit(ctx->M, dt);
     A.max_lanes = 32;
     // Recording an ended walk and refilling its lane costs the warp about 300
     // instructions, however many lanes take part; a lane that waits idles.
@@ -2172,7 +2192,7 @@ extern "C" sdd_status sdd_batch_values(const sdd_batch_entry *entries, int32_t n
         B.tpool = c->M.tpool;
         B.K = c->K;
         for (int k = 0; k < c->E * c->K; ++k) B.kappa[k] = c->M.kappa[k];
-        for (int k = 0; k < c->E; ++k) B.ev[k] = c->M.ev[k];
+        fill_samples(B, c->M, dt);
     }
     cudaStream_t s = own->stream;
     const size_t ob = (size_t)n_nodes * own->E * 2 * sizeof(double);
@@ -2192,6 +2212,7 @@ extern "C" sdd_status sdd_batch_values(const sdd_batch_entry *entries, int32_t n
     A.nodes = (const double *)own->nodes.p;
     A.node_ids = (const uint32_t *)own->node_ids.p;
     A.models = (const BatchModel *)own->batch_models.p;
+    A.turns = std::all_of(table.begin(), table.end(), [](const BatchModel &B) { return B.turns != 0; });
     st = run(own, P, L, A, s, true, true, (double *)own->mean.p, (double *)own->se.p, n_nodes, &Mb);
     if (st != SDD_OK) return st;
     std::vector<double> hm(ob / sizeof(double)), hs(ob / sizeof(double));
@@ -2315,10 +2336,15 @@ struct sdd_server {
 
 namespace {
 
+// What a request is charged for its rates and boundary constants (the phase
+// tables made from them for a launch are not charged).
+constexpr int64_t kModelCharge = sizeof(BatchModel) - sizeof(BatchModel::turn_frac) - sizeof(BatchModel::turn_whole) +
+                                 kMaxE * (sizeof(EvalDev) - sizeof(EvalF));
+
 int64_t request_bytes(const sdd_server *srv, int32_t n_nodes) {
     const int E = srv->cfg.n_eval;
     return (int64_t)srv->slot_bytes + (int64_t)n_nodes * (16 + 4 + 8 + 8 + 32 * E) +
-           (int64_t)sizeof(BatchModel);
+           kModelCharge;
 }
 
 // Walks a launch gets through per second, for the virtual deadlines below
@@ -2454,6 +2480,7 @@ sdd_status srv_launch(sdd_server *srv, SrvLane &L, std::vector<SrvPiece> &batch)
     A.queue = (int32_t *)L.queue.p;
     A.error = (int32_t *)L.err.p;
     A.models = (const BatchModel *)L.models.p;
+    A.turns = std::all_of(table.begin(), table.end(), [](const BatchModel &B) { return B.turns != 0; });
     ModelDev Mb = srv->tmpl->M;
     Mb.gcode = GC_RASTER_MULTI;
     Mb.K = Kmax;
@@ -2759,7 +2786,7 @@ extern "C" sdd_status sdd_server_submit(sdd_server *srv, const sdd_request_desc 
     r->K = m->n_materials;
     r->bm.K = m->n_materials;
     for (int k = 0; k < md.E * md.K; ++k) r->bm.kappa[k] = md.kappa[k];
-    for (int k = 0; k < md.E; ++k) r->bm.ev[k] = md.ev[k];
+    fill_samples(r->bm, md, srv->cfg.dt);
     const int n = req->n_nodes, E = c.n_eval;
     r->nodes.assign(req->nodes_xz, req->nodes_xz + 2 * n);
     r->ids.resize(n);

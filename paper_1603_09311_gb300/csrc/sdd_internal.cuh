@@ -5,6 +5,7 @@
 // walk compiled without FMA contraction).
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <vector>
 
@@ -100,14 +101,52 @@ __host__ __device__ constexpr int tile_cols(int n) { return n / kTile + 2; }
 // exact below 2^22.
 constexpr int kMaxRasterSide = 1 << 20;
 
+// Phase of a unit of occupation: kappa dt / (4 pi) turns, the fraction in
+// units of 2^-64 turns and the whole turns.  The phase of a walk is then a sum
+// of integer products modulo a turn, exact but for the fractions' rounding
+// (2^-53 of kappa dt, as a double has).  For kappa dt / (4 pi) below
+// kMaxTurns only.
+constexpr double kMaxTurns = 1048576.0;
+struct PhaseTurn {
+    uint64_t frac;
+    uint32_t whole;
+};
+__host__ __device__ inline PhaseTurn phase_turn(double kappa, double dt) {
+    const double t = kappa * dt * 0.07957747154594767;
+    const double w = floor(t);
+    PhaseTurn p;
+    p.frac = (uint64_t)((t - w) * 18446744073709551616.0);
+    p.whole = (uint32_t)w;
+    return p;
+}
+
+// The boundary constants of an evaluation as the single-precision samples use
+// them: column wavenumbers, left corner values and right less left.
+struct EvalF {
+    float kl_re, kl_im, kr_re, kr_im;
+    float tl_re, tl_im, td_re, td_im;
+    float bl_re, bl_im, bd_re, bd_im;
+};
+__host__ __device__ inline EvalF eval_f(const EvalDev &E) {
+    EvalF f;
+    f.kl_re = (float)E.kl_re; f.kl_im = (float)E.kl_im; f.kr_re = (float)E.kr_re; f.kr_im = (float)E.kr_im;
+    f.tl_re = (float)E.tl_re; f.tl_im = (float)E.tl_im;
+    f.td_re = (float)(E.tr_re - E.tl_re); f.td_im = (float)(E.tr_im - E.tl_im);
+    f.bl_re = (float)E.bl_re; f.bl_im = (float)E.bl_im;
+    f.bd_re = (float)(E.br_re - E.bl_re); f.bd_im = (float)(E.br_im - E.bl_im);
+    return f;
+}
+
 // Per-model data of a batched launch (device memory).
 struct BatchModel {
     const int8_t *raster;
     const uint32_t *tcoarse;
     const uint8_t *tpool;
-    int32_t K, pad;
+    int32_t K, turns;             // turns: the phases fit PhaseTurn
     double kappa[kMaxE * kMaxK];  // [E][K] of this model
-    EvalDev ev[kMaxE];
+    EvalF ev[kMaxE];
+    uint64_t turn_frac[kMaxE * kMaxK];   // PhaseTurn of each kappa at the launch's dt
+    uint32_t turn_whole[kMaxE * kMaxK];
 };
 
 struct ModelDev {
@@ -167,6 +206,7 @@ struct WalkArgs {
     uint32_t key0, key1;       // Philox key (seed)
     uint32_t rk0[10], rk1[10]; // the key of each Philox round (key bumped by the Weyl constants)
     uint32_t max_steps;
+    int32_t turns;             // single precision: every kappa dt / (4 pi) is below kMaxTurns
     int32_t exit_batch;        // ended walks of a warp recorded together (1 .. 32)
     int32_t max_lanes;         // walks of a warp at a time (1 .. 32)
     double *slots;             // [n_items][E][4]: sum re, sum im, sum re^2, sum im^2

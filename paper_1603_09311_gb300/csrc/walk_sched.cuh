@@ -166,10 +166,16 @@ struct WarpState {
 
 // The model's rates [E][K] and boundary constants [E], staged in shared
 // memory ahead of the warps' areas; sized by the model's E and K.
+// The TE walk in single precision keeps its phases as turns and its boundary
+// constants as floats there instead, in the same space.
 struct SharedTables {
     double *kappa;
     EvalDev *ev;
+    uint64_t *turn_frac;   // [E][K]
+    EvalF *evf;            // [E]
+    uint32_t *turn_whole;  // [E][K]
 };
+static_assert(sizeof(EvalF) + kMaxK * sizeof(uint32_t) <= sizeof(EvalDev), "turn tables exceed the boundary table");
 
 __host__ __device__ constexpr size_t tables_bytes(int E, int K) {
     return ((size_t)E * K * sizeof(double) + 15) / 16 * 16 + (size_t)E * sizeof(EvalDev);
@@ -231,8 +237,21 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
     Ring<W> &R = WS.ring;
     WarpState &S = WS.st;
 
-    for (int i = threadIdx.x; i < M.E * M.K; i += blockDim.x) T.kappa[i] = M.kappa[i];
-    for (int i = threadIdx.x; i < M.E; i += blockDim.x) T.ev[i] = M.ev[i];
+    T.turn_frac = reinterpret_cast<uint64_t *>(T.kappa);
+    T.evf = reinterpret_cast<EvalF *>(T.ev);
+    T.turn_whole = reinterpret_cast<uint32_t *>(T.evf + M.E);
+    if constexpr (W::kTurns) {
+        if (A.turns)
+            for (int i = threadIdx.x; i < M.E * M.K; i += blockDim.x) {
+                const PhaseTurn p = phase_turn(M.kappa[i], A.dt);
+                T.turn_frac[i] = p.frac;
+                T.turn_whole[i] = p.whole;
+            }
+        for (int i = threadIdx.x; i < M.E; i += blockDim.x) T.evf[i] = eval_f(M.ev[i]);
+    } else {
+        for (int i = threadIdx.x; i < M.E * M.K; i += blockDim.x) T.kappa[i] = M.kappa[i];
+        for (int i = threadIdx.x; i < M.E; i += blockDim.x) T.ev[i] = M.ev[i];
+    }
 
     const int lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
@@ -262,84 +281,122 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
     int model = 0;
     uint32_t path = 0;
 
-    // Turn records [head, head + cnt) of the ring into samples; lane l
-    // handles evaluation l mod Epad of records l / Epad, l / Epad + 32 / Epad,
-    // ...; the samples of each item are summed across the lanes in a fixed
-    // shuffle order and lane e adds them to the item's slot for evaluation e.
+    // The record of ring entry s as its sample for evaluation e (zero for a
+    // truncated walk, or when the records are dumped: then written out).
+    auto take = [&](int s, int e) {
+        const uint32_t meta = R.meta[s];
+        const bool tr = (meta >> 6) & 1u;
+        typename W::Occ c[KMAX];
+        if constexpr (W::kStored == KMAX) {
+#pragma unroll
+            for (int j = 0; j < KMAX; ++j) c[j] = R.cnt[j][s];
+        } else {
+            uint32_t rest = R.n[s];
+#pragma unroll
+            for (int j = 1; j < KMAX; ++j) {
+                c[j] = R.cnt[j - 1][s];
+                rest -= c[j];
+            }
+            c[0] = rest;
+        }
+        if (dump) {
+            if (e == 0) {
+                const int64_t o = (int64_t)(R.path[s] - A.items[0].path0);
+                double ex, ez;
+                W::to_abs(M, R.x[s], R.z[s], ex, ez);
+                A.rec_steps[o] = (int64_t)R.n[s] + (tr ? 0 : 1);
+#pragma unroll
+                for (int j = 0; j < KMAX; ++j)
+                    if (j < M.K) {
+                        if (A.rec_counts) A.rec_counts[o * M.K + j] = (int64_t)c[j];
+                        if (A.rec_occ) A.rec_occ[o * M.K + j] = (double)c[j];
+                    }
+                if (A.rec_hits) A.rec_hits[o] = (int64_t)R.aux[s];
+                A.rec_exit[3 * o + 0] = ex;
+                A.rec_exit[3 * o + 1] = ez;
+                A.rec_exit[3 * o + 2] = (double)R.th[s];
+                A.rec_wall[o] = tr ? -1 : (int)(meta & 3u);
+                A.rec_mlast[o] = (int)((meta >> 2) & 7u);
+            }
+            return make_double2(0.0, 0.0);
+        }
+        if (tr) return make_double2(0.0, 0.0);
+        return W::sample(M, T, A, (int)(meta >> 8), e, R.x[s], R.z[s], R.th[s], (int)(meta & 3u),
+                         (int)((meta >> 2) & 7u), c);
+    };
+
+    // Add the sums q (re, im, re^2, im^2) of the lanes of each evaluation to
+    // item it's slots, in a fixed order.  Lanes e, e + Epad, ... hold
+    // evaluation e; a level of the sum halves the values a lane carries while
+    // it can, so 32 lanes of one evaluation take 6 additions, not 20.
+    auto add_slots = [&](int it, double q0, double q1, double q2, double q3) {
+        const int Epad = M.Epad, my_e = lane & (Epad - 1);
+        double *o = A.slots + ((size_t)it * M.E + my_e) * 4;
+        if (Epad <= 16) {
+            const bool up = lane & 16;
+            const double g0 = __shfl_xor_sync(kFull, up ? q0 : q2, 16), g1 = __shfl_xor_sync(kFull, up ? q1 : q3, 16);
+            q0 = (up ? q2 : q0) + g0;
+            q1 = (up ? q3 : q1) + g1;
+            if (up) o += 2;
+        }
+        if (Epad <= 8) {
+            const bool up = lane & 8;
+            const double g = __shfl_xor_sync(kFull, up ? q0 : q1, 8);
+            q0 = (up ? q1 : q0) + g;
+            if (up) o += 1;
+        }
+        for (int off = 4; off >= Epad; off >>= 1) q0 += __shfl_xor_sync(kFull, q0, off);
+        if (my_e >= M.E || (lane & 7 & ~(Epad - 1)) != 0) return;
+        o[0] += q0;
+        if (Epad > 8) o[1] += q1;
+        if (Epad > 16) {
+            o[2] += q2;
+            o[3] += q3;
+        }
+    };
+
+    // Turn records [head, head + cnt) of the ring (cnt <= 32) into samples,
+    // 32 / Epad records a round; lane l handles evaluation l mod Epad.  Up to 4
+    // evaluations: all records in ring order, then the sums of each item in
+    // the round.  More: item by item, a lane adding up its samples over the
+    // item's rounds first, so that the item's slots are touched once.
     auto process = [&](int cnt) {
-        const int Epad = M.Epad;
-        const int my_e = lane & (Epad - 1);
-        const int my_ro = lane / Epad;
-        const int per_round = 32 / Epad;
         const uint32_t head = S.head;
-        const int rounds = (cnt * Epad + 31) >> 5;
-        for (int k = 0; k < rounds; ++k) {
-            const int ri = k * per_round + my_ro;
-            double2 v = make_double2(0.0, 0.0);
-            int my_it = -1;
-            if (ri < cnt && my_e < M.E) {
-                const int s = (head + ri) & (kRing - 1);
-                const uint32_t meta = R.meta[s];
-                const bool tr = (meta >> 6) & 1u;
-                typename W::Occ c[KMAX];
-                if constexpr (W::kStored == KMAX) {
-#pragma unroll
-                    for (int j = 0; j < KMAX; ++j) c[j] = R.cnt[j][s];
+        const int Epad = M.Epad, my_e = lane & (Epad - 1);
+        const int per_round = 32 / Epad, my_ro = lane / Epad;
+        const int rec_it = lane < cnt ? R.item[(head + lane) & (kRing - 1)] : -1;
+        unsigned pend = kFull >> (32 - cnt);
+        while (pend) {
+            const int it = __shfl_sync(kFull, rec_it, __ffs(pend) - 1);
+            const unsigned sel = Epad <= 4 ? pend : __ballot_sync(kFull, rec_it == it);
+            double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+            for (unsigned left = sel; left;) {
+                // this round's records: the lowest per_round bits of left
+                unsigned m = left;
+                for (int j = 0; j < my_ro; ++j) m &= m - 1u;
+                double2 v = make_double2(0.0, 0.0);
+                const int at = __ffs(m) - 1;
+                if (m && my_e < M.E) v = take((head + at) & (kRing - 1), my_e);
+                if (Epad <= 4) {
+                    const int my_it = __shfl_sync(kFull, rec_it, at & 31);
+                    unsigned todo = dump ? 0u : __ballot_sync(kFull, m != 0u);
+                    while (todo) {
+                        const int one = __shfl_sync(kFull, my_it, __ffs(todo) - 1);
+                        const bool mine = m != 0u && my_it == one;
+                        const double b0 = mine ? v.x : 0.0, b1 = mine ? v.y : 0.0;
+                        add_slots(one, b0, b1, b0 * b0, b1 * b1);
+                        todo &= ~__ballot_sync(kFull, mine);
+                    }
                 } else {
-                    uint32_t rest = R.n[s];
-#pragma unroll
-                    for (int j = 1; j < KMAX; ++j) {
-                        c[j] = R.cnt[j - 1][s];
-                        rest -= c[j];
-                    }
-                    c[0] = rest;
+                    a0 += v.x;
+                    a1 += v.y;
+                    a2 = fma(v.x, v.x, a2);
+                    a3 = fma(v.y, v.y, a3);
                 }
-                if (dump) {
-                    if (my_e == 0) {
-                        const int64_t o = (int64_t)(R.path[s] - A.items[0].path0);
-                        double ex, ez;
-                        W::to_abs(M, R.x[s], R.z[s], ex, ez);
-                        A.rec_steps[o] = (int64_t)R.n[s] + (tr ? 0 : 1);
-#pragma unroll
-                        for (int j = 0; j < KMAX; ++j)
-                            if (j < M.K) {
-                                if (A.rec_counts) A.rec_counts[o * M.K + j] = (int64_t)c[j];
-                                if (A.rec_occ) A.rec_occ[o * M.K + j] = (double)c[j];
-                            }
-                        if (A.rec_hits) A.rec_hits[o] = (int64_t)R.aux[s];
-                        A.rec_exit[3 * o + 0] = ex;
-                        A.rec_exit[3 * o + 1] = ez;
-                        A.rec_exit[3 * o + 2] = (double)R.th[s];
-                        A.rec_wall[o] = tr ? -1 : (int)(meta & 3u);
-                        A.rec_mlast[o] = (int)((meta >> 2) & 7u);
-                    }
-                } else if (!tr) {
-                    v = W::sample(M, T, A, (int)(meta >> 8), my_e, R.x[s], R.z[s], R.th[s],
-                                  (int)(meta & 3u), (int)((meta >> 2) & 7u), c);
-                    my_it = R.item[s];
-                }
+                for (int j = 0; j < per_round; ++j) left &= left - 1u;
             }
-            unsigned pend = __ballot_sync(kFull, my_it >= 0);
-            while (pend) {
-                const int it = __shfl_sync(kFull, my_it, __ffs(pend) - 1);
-                const bool mine = my_it == it;
-                double a0 = mine ? v.x : 0.0, a1 = mine ? v.y : 0.0;
-                double a2 = a0 * a0, a3 = a1 * a1;
-                for (int off = 16; off >= Epad; off >>= 1) {
-                    a0 += __shfl_xor_sync(kFull, a0, off);
-                    a1 += __shfl_xor_sync(kFull, a1, off);
-                    a2 += __shfl_xor_sync(kFull, a2, off);
-                    a3 += __shfl_xor_sync(kFull, a3, off);
-                }
-                if (lane < M.E) {
-                    double *o = A.slots + ((size_t)it * M.E + lane) * 4;
-                    o[0] += a0;
-                    o[1] += a1;
-                    o[2] += a2;
-                    o[3] += a3;
-                }
-                pend &= ~__ballot_sync(kFull, mine);
-            }
+            if (Epad > 4 && !dump) add_slots(it, a0, a1, a2, a3);
+            pend &= ~sel;
         }
         __syncwarp();
         S.head = head + (uint32_t)cnt;
@@ -433,8 +490,7 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
         }
     };
 
-    // Records of the walks that have ended (st: 1 exited, 2 truncated), then
-    // a batch of samples once 32 records are waiting.
+    // Records of the walks that have ended (st: 1 exited, 2 truncated).
     ExitInfo<Real> ei{};
     auto on_exits = [&](int st) {
         const unsigned em = __ballot_sync(kFull, st != 0);
@@ -467,32 +523,35 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
             S.trunc += (unsigned long long)__popc(trm);
         }
         __syncwarp();
-        while (S.tail - S.head >= 32) process(32);
     };
 
+    // The rest of an exit: records, refill, and samples once 32 records are
+    // waiting, or at the end.
+    int n_live = 0;
+    auto settle = [&](int ended) {
+        on_exits(ended);
+        refill();
+        n_live = __popc(__ballot_sync(kFull, active));
+        while (S.tail - S.head >= 32 || (n_live == 0 && S.tail != S.head)) process((int)min(S.tail - S.head, 32u));
+    };
     refill();
-    int n_live = __popc(__ballot_sync(kFull, active));  // lanes with a walk, ended ones included
-    // A lane whose walk has ended waits (ended != 0) until exit_batch lanes of
-    // the warp have, or all of them: the records and the refill cost a warp
-    // the same for one ended walk as for several.
-    int ended = 0;
+    n_live = __popc(__ballot_sync(kFull, active));
+
+    // One walk a lane.  A lane whose walk has ended waits until exit_batch
+    // lanes of the warp have, or all of them: the records and the refill cost
+    // a warp the same for one ended walk as for several.
     if constexpr (W::kAlone) {
-        int n_batch = min(n_live, A.exit_batch);
         while (n_live > 0) {
             if (W::kCoop && n_live <= kCoopWalks &&
                 (A.max_lanes <= kCoopWalks || (S.queue_empty && S.disp_rem == 0)))
                 break;
+            const int n_batch = min(n_live, A.exit_batch);
             int st = active ? 0 : -1;
             do {
                 if (st == 0) st = w.iterate(M, A, path, ei);
             } while (__popc(__ballot_sync(kFull, st > 0)) < n_batch);
-            ended = max(st, 0);
             active = st == 0;
-            on_exits(ended);
-            ended = 0;
-            refill();
-            n_live = __popc(__ballot_sync(kFull, active));
-            n_batch = min(n_live, A.exit_batch);
+            settle(max(st, 0));
         }
     }
 
@@ -501,57 +560,56 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
     // random words, the normals, the move, the tests).  Here each walk gets
     // 32 / a lanes, two steps a lane and round: the words, the normals and the
     // tests of all its steps are formed side by side, and only the moves
-    // remain one after the other.  The lanes work for the same walks until
-    // one of them ends.
+    // remain one after the other.  The lanes work for the same walks until one
+    // of them ends.
     if constexpr (W::kCoop) {
         while (n_live > 0) {
-            const unsigned act = __ballot_sync(kFull, active);
-            const int per = 32 / n_live;
-            const int j = lane / per;
-            const uint32_t q = (uint32_t)(lane % per);
-            const bool in = j < n_live;
-            unsigned m = act;
-            for (int t = 0; t < j && in; ++t) m &= m - 1u;
-            const int owner = __ffs(m) - 1;
-            const unsigned seg = in ? (kFull >> (32 - per)) << (j * per) : 0u;
-            const int last = in ? j * per + per - 1 : lane;
-            typename W::CoopInc *buf = WS.coop + (in ? j * 2 * per : 0);
-            typename W::Coop c;
-            w.coop_begin(c, owner, lane);
-            int code;
-            unsigned events;
-            for (;;) {
-                code = W::coop_round(M, A, c, buf, q, per, in);
-                events = __ballot_sync(kFull, code != 0);
-                if (events) break;
-                W::coop_count(M, c, in ? 2 : 0);
-                w.coop_next(c, per, last);
+            int ended = 0;  // the lane's walk: 1 exited, 2 truncated
+            do {
+                const unsigned act = __ballot_sync(kFull, active);
+                const int per = 32 / n_live;
+                const int j = lane / per;
+                const uint32_t q = (uint32_t)(lane % per);
+                const bool in = j < n_live;
+                unsigned m = act;
+                for (int t = 0; t < j && in; ++t) m &= m - 1u;
+                const int owner = __ffs(m) - 1;
+                const unsigned seg = in ? (kFull >> (32 - per)) << (j * per) : 0u;
+                const int last = in ? j * per + per - 1 : lane;
+                typename W::CoopInc *buf = WS.coop + (in ? j * 2 * per : 0);
+                typename W::Coop c;
+                w.coop_begin(c, owner, lane);
+                int code;
+                unsigned events;
+                for (;;) {
+                    code = W::coop_round(M, A, c, buf, q, per, in);
+                    events = __ballot_sync(kFull, code != 0);
+                    if (events) break;
+                    W::coop_count(M, c, in ? 2 : 0);
+                    w.coop_next(c, per, last);
+                    __syncwarp();
+                }
+                // the steps before the segment's first event count (of the
+                // event's lane: those before it)
+                const int first = (events & seg) ? __ffs(events & seg) - 1 : 32;
+                const int base = __popc(act & lt_mask) * per & 31;  // this lane's walk, if it owns one
+                if constexpr (W::kEvents) {
+                    ended = w.coop_events(M, A, c, code, first, per, active ? base : 0, active, ei);
+                } else {
+                    W::coop_count(M, c, !in || lane > first ? 0 : (lane < first ? 2 : (code == 3 ? 2 : code - 1)));
+                    if (lane == first) w.coop_put(c, code, q, lane);
+                    const int fcode = __shfl_sync(kFull, code, first & 31);
+                    const int my_st = first == 32 ? 0 : (fcode == 3 ? 2 : 1);
+                    const int st_own = __shfl_sync(kFull, my_st, base);
+                    w.coop_end(c, seg, per, active ? base : 0, active);
+                    ended = active ? st_own : 0;
+                }
                 __syncwarp();
-            }
-            // the steps before the segment's first event count (of the event's
-            // lane: those before it)
-            const int first = (events & seg) ? __ffs(events & seg) - 1 : 32;
-            const int base = __popc(act & lt_mask) * per & 31;  // this lane's walk, if it owns one
-            if constexpr (W::kEvents) {
-                ended = w.coop_events(M, A, c, code, first, per, active ? base : 0, active, ei);
-                if (__ballot_sync(kFull, ended != 0) == 0) continue;
-            } else {
-                W::coop_count(M, c, !in || lane > first ? 0 : (lane < first ? 2 : (code == 3 ? 2 : code - 1)));
-                if (lane == first) w.coop_put(c, code, q, lane);
-                const int fcode = __shfl_sync(kFull, code, first & 31);
-                const int my_st = first == 32 ? 0 : (fcode == 3 ? 2 : 1);
-                const int st_own = __shfl_sync(kFull, my_st, base);
-                w.coop_end(c, seg, per, active ? base : 0, active);
-                ended = active ? st_own : 0;
-            }
+            } while (__ballot_sync(kFull, ended != 0) == 0);
             if (ended) active = false;
-            __syncwarp();
-            on_exits(ended);
-            refill();
-            n_live = __popc(__ballot_sync(kFull, active));
+            settle(ended);
         }
     }
-    if (S.tail != S.head) process((int)(S.tail - S.head));
     // every item handed to this warp has been flushed (its walks all ended)
 
     unsigned long long my_steps = S.steps[lane];

@@ -138,3 +138,41 @@ def test_few_tm_walks_equal_the_walks_of_a_large_launch(name, x0, max_steps):
             _same(rec(n, block_threads=32, ctas_per_sm=1), big, n)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("E", [1, 2, 3, 4, 5, 8, 9, 16, 17, 32])
+def test_sums_of_several_evaluations_equal_each_alone(E):
+    # the walks do not depend on the rates, so row e of E evaluations is the
+    # evaluation alone; only the order of the FP64 sums differs (500 terms)
+    kap = np.stack([np.zeros(E), np.geomspace(0.1, 200.0, E), np.geomspace(50.0, 0.3, E)], axis=1)
+    model = dict(I.quarterspace(), kappa=kap)
+    nodes, paths = I.nodes_line((0.0, 0.1), (0.0, 0.8), 3), np.array([500, 33, 470])
+    ctx = sdd.sdd_create(model)
+    mean, se, _ = sdd.sdd_interface_values(ctx, nodes, paths, 1e-3, 4)
+    ctx.close()
+    for e in {0, E // 2, E - 1}:
+        one = sdd.sdd_create(dict(model, kappa=kap[e:e + 1]))
+        m1, s1, _ = sdd.sdd_interface_values(one, nodes, paths, 1e-3, 4)
+        one.close()
+        assert np.abs(mean[:, e] - m1[:, 0]).max() <= 1e-13 and np.abs(se[:, e] - s1[:, 0]).max() <= 1e-13
+
+
+@pytest.mark.parametrize("dt", [1e-3, 2e-2])
+def test_phases_in_turns_equal_the_phases_in_doubles(dt):
+    # a rate too large for the integer phases (kappa dt / 4 pi >= 2^20) puts the
+    # whole model on the FP64 sum; the other rows must agree: the two phases
+    # differ by about 1e-13, so at most a sample in 1e5 rounds to another float
+    # (1.2e-7): 1e-9 of |g| <= 1 for 900 walks.  At dt = 0.02 the larger rates
+    # turn more than once a step.
+    rows = [[0.0, 0.7, 3.0], [0.0, 2000.0, 1.0e4], [0.0, 900.0, 0.01]]
+    nodes = I.nodes_line((0.0, 0.1), (0.0, 0.8), 2)
+    got = []
+    for extra in ([], [[0.0, 5.0, 2.0e7 / dt]]):
+        ctx = sdd.sdd_create(dict(I.quarterspace(), kappa=rows + extra, g=("affine", 1.0, 0.3, 0.2)))
+        got.append(sdd.sdd_interface_values(ctx, nodes, 900, dt, 4)[0][:, :3])
+        ctx.close()
+    assert np.abs(got[0] - got[1]).max() <= 1e-9
+    ref = O.interface_values(dict(I.quarterspace(), kappa=rows, g=("affine", 1.0, 0.3, 0.2)), nodes, 900, dt, 4, urule=23)
+    # the first row's rates are small: a step counted in the neighbouring
+    # material is a phase of 1.2 dt in one of 900 walks
+    assert np.abs(got[0][:, 0] - ref["mean"][:, 0]).max() <= 1e-4
