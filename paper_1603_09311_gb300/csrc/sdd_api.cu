@@ -132,7 +132,7 @@ struct sdd_ctx {
     int geo = GEO_SHAPES;
     DevBuf raster, tiles;
     // per-call scratch
-    DevBuf items, slots, trunc, counters, queue, err, nodes, node_ids, mean, se;
+    DevBuf items, slots, trunc, counters, err, nodes, node_ids, mean, se;  // counters: and the queue heads
     DevBuf rec_steps, rec_counts, rec_occ, rec_hits, rec_exit, rec_wall, rec_mlast;
     DevBuf batch_models;  // model table of batched launches owned by this context
     DevBuf red_index;     // node -> first range of the range reduction (sdd_reduce_sums)
@@ -419,11 +419,15 @@ constexpr int kReduceThreads = 128;  // 4 (node, evaluation) pairs a CTA
 inline unsigned reduce_ctas(long long pairs) { return (unsigned)((pairs * 32 + kReduceThreads - 1) / kReduceThreads); }
 
 // Per node and evaluation (one warp): the sums of its items, then the mean
-// and the standard errors of the real and imaginary parts.
+// and the standard errors of the real and imaginary parts.  counters_out
+// (nullable): the caller's copy of the walk's counters, taken along here (as a
+// copy of its own behind the launch it took 2 us of a 60 us call).
 __global__ void __launch_bounds__(kReduceThreads)
     reduce_kernel(const double *__restrict__ slots, const int32_t *__restrict__ trunc,
                   const Item *__restrict__ items, const int32_t *__restrict__ node_item0, int n_nodes, int E,
-                  double *__restrict__ mean, double *__restrict__ se) {
+                  double *__restrict__ mean, double *__restrict__ se, const unsigned long long *counters,
+                  unsigned long long *counters_out) {
+    if (counters_out && blockIdx.x == 0 && threadIdx.x < 3) counters_out[threadIdx.x] = counters[threadIdx.x];
     const int t = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (t >= n_nodes * E) return;
     const int j = t / E, e = t % E, lane = threadIdx.x & 31;
@@ -882,6 +886,11 @@ void table_args(const Plan &P, int n_nodes, const unsigned char *d, WalkArgs &A)
     A.n_queues = P.qbase.empty() ? 1 : (int32_t)P.qbase.size() - 1;
 }
 
+// The walk's counters (3 x u64) and, behind them, its queue heads: one block,
+// cleared by one memset.
+constexpr size_t kQueueOff = 32;
+size_t counter_bytes(const Plan &P) { return kQueueOff + std::max<size_t>(P.qbase.size(), 1) * sizeof(int32_t); }
+
 sdd_status prepare(sdd_ctx *ctx, const Plan &P, int n_nodes, cudaStream_t s) {
     const size_t ni = P.items.size();
     if (ni == 0) return SDD_OK;
@@ -889,8 +898,7 @@ sdd_status prepare(sdd_ctx *ctx, const Plan &P, int n_nodes, cudaStream_t s) {
     SDD_CUDA(ctx->items.ensure(hbytes));
     SDD_CUDA(ctx->slots.ensure(ni * (size_t)ctx->E * 4 * sizeof(double)));
     SDD_CUDA(ctx->trunc.ensure(ni * sizeof(int32_t)));
-    SDD_CUDA(ctx->counters.ensure(3 * sizeof(unsigned long long)));
-    SDD_CUDA(ctx->queue.ensure(std::max<size_t>(P.qbase.size(), 1) * sizeof(int32_t)));
+    SDD_CUDA(ctx->counters.ensure(counter_bytes(P)));
     SDD_CUDA(ctx->err.ensure(sizeof(int32_t)));
     ctx->last_h2d = 0;
     const bool own = &P == &ctx->plan;
@@ -915,12 +923,11 @@ sdd_status prepare(sdd_ctx *ctx, const Plan &P, int n_nodes, cudaStream_t s) {
 // Device work of a prepared plan: clear counters, walk, reduce.
 sdd_status enqueue(sdd_ctx *ctx, const Plan &P, const Launch &L, WalkArgs A, cudaStream_t s,
                    bool timed, bool do_reduce, double *d_mean, double *d_se, int n_nodes,
-                   const ModelDev *model = nullptr) {
+                   const ModelDev *model = nullptr, uint64_t *d_counters = nullptr) {
     const ModelDev &MD = model ? *model : ctx->M;
     const size_t ni = P.items.size();
     if (ni == 0) return SDD_OK;
-    SDD_CUDA(cudaMemsetAsync(ctx->queue.p, 0, std::max<size_t>(P.qbase.size(), 1) * sizeof(int32_t), s));
-    SDD_CUDA(cudaMemsetAsync(ctx->counters.p, 0, 3 * sizeof(unsigned long long), s));
+    SDD_CUDA(cudaMemsetAsync(ctx->counters.p, 0, counter_bytes(P), s));
     A.items = (const Item *)ctx->items.p;
     A.n_items = (int32_t)ni;
     A.max_lanes = P.qbase.empty() ? warp_lanes(P.total_paths, L) : 32;
@@ -928,7 +935,7 @@ sdd_status enqueue(sdd_ctx *ctx, const Plan &P, const Launch &L, WalkArgs A, cud
     A.slots = (double *)ctx->slots.p;
     A.item_trunc = (int32_t *)ctx->trunc.p;
     A.counters = (unsigned long long *)ctx->counters.p;
-    A.queue = (int32_t *)ctx->queue.p;
+    A.queue = reinterpret_cast<int32_t *>(static_cast<unsigned char *>(ctx->counters.p) + kQueueOff);
     A.error = (int32_t *)ctx->err.p;
     const int warps_per_cta = L.block / 32;
     int grid = L.grid;
@@ -945,7 +952,8 @@ sdd_status enqueue(sdd_ctx *ctx, const Plan &P, const Launch &L, WalkArgs A, cud
         const int32_t *d_i0 = (const int32_t *)(reinterpret_cast<unsigned char *>(ctx->items.p) + ni * sizeof(Item));
         reduce_kernel<<<reduce_ctas(nt), kReduceThreads, 0, s>>>((const double *)ctx->slots.p,
                                                       (const int32_t *)ctx->trunc.p, d_items, d_i0,
-                                                      n_nodes, ctx->E, d_mean, d_se);
+                                                      n_nodes, ctx->E, d_mean, d_se, A.counters,
+                                                      reinterpret_cast<unsigned long long *>(d_counters));
         SDD_CUDA(cudaGetLastError());
     }
     return SDD_OK;
@@ -953,10 +961,10 @@ sdd_status enqueue(sdd_ctx *ctx, const Plan &P, const Launch &L, WalkArgs A, cud
 
 sdd_status run(sdd_ctx *ctx, const Plan &P, const Launch &L, WalkArgs A, cudaStream_t s,
                bool timed, bool do_reduce, double *d_mean, double *d_se, int n_nodes,
-               const ModelDev *model = nullptr) {
+               const ModelDev *model = nullptr, uint64_t *d_counters = nullptr) {
     sdd_status st = prepare(ctx, P, n_nodes, s);
     if (st != SDD_OK) return st;
-    return enqueue(ctx, P, L, A, s, timed, do_reduce, d_mean, d_se, n_nodes, model);
+    return enqueue(ctx, P, L, A, s, timed, do_reduce, d_mean, d_se, n_nodes, model, d_counters);
 }
 
 }  // namespace
@@ -1080,7 +1088,7 @@ sdd_status sdd_create(const sdd_model_desc *model, sdd_ctx **out) {
 void sdd_destroy(sdd_ctx *c) {
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
-    DevBuf *bufs[] = {&c->raster, &c->tiles, &c->items, &c->slots, &c->trunc, &c->counters, &c->queue,
+    DevBuf *bufs[] = {&c->raster, &c->tiles, &c->items, &c->slots, &c->trunc, &c->counters,
                       &c->err, &c->nodes, &c->node_ids, &c->mean, &c->se, &c->rec_steps,
                       &c->rec_counts, &c->rec_occ, &c->rec_hits, &c->rec_exit, &c->rec_wall,
                       &c->rec_mlast,
@@ -1217,14 +1225,8 @@ sdd_status sdd_interface_values_device(sdd_ctx *ctx, const double *d_nodes_xz,
     WalkArgs A = base_args(ctx, L, dt, seed);
     A.nodes = d_nodes_xz;
     A.node_ids = d_node_ids;
-    if (!(cfg && cfg->use_graph)) {
-        st = run(ctx, P, L, A, s, false, true, d_mean, d_se, n_nodes);
-        if (st != SDD_OK) return st;
-        if (d_counters)
-            SDD_CUDA(cudaMemcpyAsync(d_counters, ctx->counters.p, 3 * sizeof(uint64_t),
-                                     cudaMemcpyDeviceToDevice, s));
-        return SDD_OK;
-    }
+    if (!(cfg && cfg->use_graph))
+        return run(ctx, P, L, A, s, false, true, d_mean, d_se, n_nodes, nullptr, d_counters);
     // graph mode: the item table goes up on the caller's stream; the device
     // work is captured on the context's stream into a graph, the cached
     // executable graph is updated in place (re-instantiated only when the
@@ -1233,12 +1235,7 @@ sdd_status sdd_interface_values_device(sdd_ctx *ctx, const double *d_nodes_xz,
     if (st != SDD_OK) return st;
     cudaGraph_t g = nullptr;
     SDD_CUDA(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-    st = enqueue(ctx, P, L, A, ctx->stream, false, true, d_mean, d_se, n_nodes);
-    if (st == SDD_OK && d_counters) {
-        cudaError_t e = cudaMemcpyAsync(d_counters, ctx->counters.p, 3 * sizeof(uint64_t),
-                                        cudaMemcpyDeviceToDevice, ctx->stream);
-        if (e != cudaSuccess) st = cuda_fail(e, "counter copy");
-    }
+    st = enqueue(ctx, P, L, A, ctx->stream, false, true, d_mean, d_se, n_nodes, nullptr, d_counters);
     cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
     if (st != SDD_OK) {
         if (g) cudaGraphDestroy(g);
@@ -1500,11 +1497,8 @@ extern "C" sdd_status sdd_interface_values_noalloc(sdd_ctx *ctx, const double *d
     const int nt = n_nodes * ctx->E;
     reduce_kernel<<<reduce_ctas(nt), kReduceThreads, 0, s>>>(
         A.slots, A.item_trunc, A.items, reinterpret_cast<const int32_t *>(base + kNaOffNodeItem0),
-        n_nodes, ctx->E, d_mean, d_se);
+        n_nodes, ctx->E, d_mean, d_se, A.counters, reinterpret_cast<unsigned long long *>(d_counters));
     SDD_CUDA(cudaGetLastError());
-    if (d_counters)
-        SDD_CUDA(cudaMemcpyAsync(d_counters, A.counters, 3 * sizeof(uint64_t),
-                                 cudaMemcpyDeviceToDevice, s));
     return SDD_OK;
 }
 
@@ -1881,7 +1875,7 @@ extern "C" sdd_status sdd_interface_values_async(sdd_ctx *ctx, const double *nod
             const int nt = n_nodes * ctx->E;
             reduce_kernel<<<reduce_ctas(nt), kReduceThreads, 0, s>>>(
                 A.slots, A.item_trunc, A.items, reinterpret_cast<const int32_t *>(r->dev + o_i0), n_nodes, ctx->E,
-                reinterpret_cast<double *>(r->dev + o_mean), reinterpret_cast<double *>(r->dev + o_se));
+                reinterpret_cast<double *>(r->dev + o_mean), reinterpret_cast<double *>(r->dev + o_se), nullptr, nullptr);
             q(cudaGetLastError(), "reduce kernel launch");
         }
         q(cudaMemcpyAsync(r->host + o_mean, r->dev + o_mean, total - o_mean, cudaMemcpyDeviceToHost, s),
