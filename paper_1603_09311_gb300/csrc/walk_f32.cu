@@ -285,11 +285,12 @@ struct WalkerF32 {
     }
     static constexpr int kPend = 6;
 
-    __device__ __forceinline__ void start(const ModelDev &M, const WalkArgs &A, double x0,
-                                          double z0, uint32_t path, uint32_t node_id, int model) {
+    __device__ __forceinline__ void start(const ModelDev &M, const WalkArgs &A, const WarpState &S, uint32_t path,
+                                          int model) {
+        const uint32_t node_id = S.nid;
         if (GC == GC_RASTER_MULTI) tco = A.models[model].tcoarse;
-        X = (float)(x0 - M.xc);
-        Z = (float)(z0 - M.zc);
+        X = S.fx0;
+        Z = S.fz0;
         dmin = fminf(M.fhw - fabsf(X), M.fhh - fabsf(Z));
         n = 0;
         occ.clear();

@@ -93,15 +93,14 @@ struct WalkerF64 {
         for (int j = 1; j < KMAX; ++j) c[j - 1] += (m == j) ? 1u : 0u;
     }
 
-    __device__ __forceinline__ void start(const ModelDev &, const WalkArgs &, double x0, double z0, uint32_t path_,
-                                          uint32_t node_id, int) {
-        x = x0;
-        z = z0;
+    __device__ __forceinline__ void start(const ModelDev &, const WalkArgs &, const WarpState &S, uint32_t path_, int) {
+        x = S.nx0;
+        z = S.nz0;
         n = 0;
 #pragma unroll
         for (int j = 0; j < kCnt; ++j) cnt[j] = 0;
         path = path_;
-        nid = node_id;
+        nid = S.nid;
     }
 
     __device__ static void place(const ModelDev &M, double x, double z, double xn, double zn,

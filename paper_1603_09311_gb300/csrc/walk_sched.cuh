@@ -156,7 +156,8 @@ struct Ring {
 struct WarpState {
     unsigned long long steps[32];
     unsigned long long walks, trunc;
-    double nx0, nz0;
+    double nx0, nz0;  // the current item's node,
+    float fx0, fz0;   // and in single-precision centred coordinates
     int32_t disp_item, disp_rem, disp_model;
     uint32_t disp_next, nid;
     uint32_t head, tail;
@@ -207,7 +208,7 @@ struct ExitInfo {
 
 // Scheduler kernel.  W is a walker type providing
 //   using Real; static constexpr int KMAX;
-//   start(M, A, x0, z0, path, node_id, model)  -- begin a walk
+//   start(M, A, S, path, model)  -- begin a walk at the warp's current node
 //   iterate(M, A, path, ExitInfo&) -> 0 running, 1 exited, 2 truncated
 //     (a few Euler steps per call; max_steps is a multiple of them)
 //   finalize(M, A, st, ExitInfo&): the exit record of a walk that has ended
@@ -263,6 +264,7 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
         S.head = S.tail = 0;
         S.queue_empty = 0;
         S.nx0 = S.nz0 = 0.0;
+        S.fx0 = S.fz0 = 0.f;
         S.home = 0;
         if (W::kGrouped && A.qbase) {
             const float x = ((float)blockIdx.x + 0.5f) / (float)gridDim.x;
@@ -461,8 +463,11 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
                     S.disp_model = I.model;
                     S.disp_next = I.path0;
                     S.disp_rem = I.count;
-                    S.nx0 = A.nodes[2 * I.node];
-                    S.nz0 = A.nodes[2 * I.node + 1];
+                    const double x0 = A.nodes[2 * I.node], z0 = A.nodes[2 * I.node + 1];
+                    S.nx0 = x0;
+                    S.nz0 = z0;
+                    S.fx0 = (float)(x0 - M.xc);
+                    S.fz0 = (float)(z0 - M.zc);
                     S.nid = A.node_ids ? A.node_ids[I.node] : (uint32_t)I.node;
                 }
                 __syncwarp();
@@ -478,7 +483,7 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
                 item = S.disp_item;
                 model = S.disp_model;
                 active = true;
-                w.start(M, A, S.nx0, S.nz0, path, S.nid, model);
+                w.start(M, A, S, path, model);
             }
             const unsigned got = __ballot_sync(kFull, mine);
             need &= ~got;

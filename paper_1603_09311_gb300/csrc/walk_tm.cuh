@@ -73,8 +73,9 @@ struct WalkerTM {
         return k;
     }
 
-    __device__ __forceinline__ void start(const ModelDev &M, const WalkArgs &A, double x0, double z0,
-                                          uint32_t path, uint32_t node_id, int) {
+    __device__ __forceinline__ void start(const ModelDev &M, const WalkArgs &A, const WarpState &S, uint32_t path, int) {
+        const double x0 = S.nx0, z0 = S.nz0;
+        const uint32_t node_id = S.nid;
         x = (Real)x0;
         z = (Real)z0;
         i = strip(M, x);
@@ -436,8 +437,9 @@ struct WalkerTM32 {
         run = 0;
     }
 
-    __device__ __forceinline__ void start(const ModelDev &M, const WalkArgs &A, double x0, double z0,
-                                          uint32_t path, uint32_t node_id, int) {
+    __device__ __forceinline__ void start(const ModelDev &M, const WalkArgs &A, const WarpState &S, uint32_t path, int) {
+        const double x0 = S.nx0, z0 = S.nz0;
+        const uint32_t node_id = S.nid;
         X = (float)x0 - M.fxc;
         Z = (float)z0 - M.fzc;
         dmin = fminf(M.fhw - fabsf(X), M.fhh - fabsf(Z));
