@@ -164,7 +164,9 @@ typedef struct {
                               node's item taking ceil(R / (guided_factor x warps)) paths,
                               R the paths not yet cut, rounded up to a multiple of 32,
                               at least 32; the queue hands them out in cut order, so
-                              they shrink toward its end.  0 = auto (tuned, else 2) */
+                              they shrink toward its end.  0 = auto (tuned, else 4).
+                              Calls of at most 16 walks a warp (64 in double
+                              precision) are cut into one share a warp instead */
 } sdd_config;
 
 typedef struct {
@@ -759,9 +761,9 @@ sdd_status sdd_model_program(const sdd_model_desc *model, int32_t *program, int3
  *   n_paths [n_nodes] host; warps >= 1; guided_factor >= 1 (guided items of
  *   about 1 / (guided_factor x warps) of the paths not yet cut, multiples of
  *   32 shrinking toward the end of the queue) used when chunk_paths == 0,
- *   else fixed items of chunk_paths paths, node by node.  (Single-precision TE
- *   calls of at most 16 walks a warp are cut into items of one share each
- *   instead, node by node: the cooperative rounds of the walk take those.)
+ *   else fixed items of chunk_paths paths, node by node.  (A launch of so few
+ *   walks that the warps share them evenly cuts items of one share instead,
+ *   node by node: see guided_factor in sdd_config.)
  *   node, path0, count [max_items] host, written in queue order; *n_items
  *   the number of items.
  * Errors: SDD_E_ARG for n_nodes < 0, a negative path count, warps < 1,

@@ -1414,15 +1414,16 @@ __global__ void noalloc_plan_kernel(int n_nodes, int chunk) {
         node_item0[n_nodes] = acc;
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < n_nodes; j += blockDim.x) {
-        int32_t it = node_item0[j];
-        for (int64_t p = 0; p < n_paths[j]; p += chunk, ++it) {
+    // a warp a node: small calls have many items of few paths
+    for (int j = threadIdx.x >> 5; j < n_nodes; j += blockDim.x >> 5) {
+        const int64_t n = n_paths[j];
+        for (int64_t k = threadIdx.x & 31, p = k * chunk; p < n; k += 32, p = k * chunk) {
             Item I;
             I.node = j;
             I.path0 = (uint32_t)p;
-            I.count = (int32_t)(n_paths[j] - p < chunk ? n_paths[j] - p : chunk);
+            I.count = (int32_t)(n - p < chunk ? n - p : chunk);
             I.model = 0;
-            items[it] = I;
+            items[node_item0[j] + k] = I;
         }
     }
 }
@@ -1455,9 +1456,11 @@ extern "C" sdd_status sdd_interface_values_noalloc(sdd_ctx *ctx, const double *d
     long long total = 0;
     for (int j = 0; j < n_nodes; ++j) total += n_paths[j];
     Launch L = choose_launch(ctx, cfg, dt);
-    // fixed-size items (the table is built on the device): about 6 per warp,
-    // widened until they fit the scratch array
+    // fixed-size items (the table is built on the device): about 6 per warp (a
+    // small call: the warps' shares), widened until they fit the scratch array
     long long chunk = L.chunk;
+    const int lanes = warp_lanes(total, L);
+    if (chunk == 0) chunk = item_share(total, L);
     if (chunk == 0) {
         const long long per = (long long)L.grid * (L.block / 32) * 6;
         chunk = std::max<long long>(32, ((total + per - 1) / per + 31) / 32 * 32);
@@ -1480,6 +1483,7 @@ extern "C" sdd_status sdd_interface_values_noalloc(sdd_ctx *ctx, const double *d
     WalkArgs A = base_args(ctx, L, dt, seed);
     A.nodes = d_nodes_xz;
     A.node_ids = d_node_ids;
+    A.max_lanes = lanes;
     A.items = reinterpret_cast<const Item *>(base + kNaOffItems);
     A.n_items = (int32_t)n_items;
     A.slots = reinterpret_cast<double *>(base + kNaOffSlots);

@@ -1,9 +1,9 @@
 // Single-precision walk (the throughput path).
 //
 // Position stepping, wall tests, material lookup and the per-walk phase
-// factor are FP32; the per-material step counts are integers; the phase sum
-// and the Monte Carlo sums are FP64.  Compiled with -ftz=true
-// -prec-div=false -prec-sqrt=false.
+// factor are FP32; the per-material step counts are integers; the phase sum is
+// in 64-bit fractions of a turn and the Monte Carlo sums are FP64.  Compiled
+// with -ftz=true -prec-div=false -prec-sqrt=false.
 //
 // One Euler-Maruyama step of Sec. 3.1 (discretised process, kappa_i = 1):
 //   (u0, u1)  two uniforms (w mod 2^23 + 1/2) 2^-23 from one Philox call,
@@ -18,6 +18,15 @@
 // distance to the nearer wall of each pair is h - |X|.  Two steps share one
 // Philox call (words 0,1 for the even step, 2,3 for the odd one), and one
 // call of iterate() runs 8 steps.
+//
+// What bounds it: instruction issue.  50 issue slots a step (64 nodes x 1e5
+// walks, dt 1e-4; 62 before the signs without flushing, one wall branch for
+// two steps and exits recorded apart) at 69 % of the issue rate, 5.4e11
+// walk-steps/s; the rest of the rate goes to the wide multiplies of Philox
+// (dispatch and math-pipe stalls, with 2.4 of 6 warps eligible on average).
+// Tried without gain: region counters on the FMA pipe (40.2 -> 40.0 ms), the
+// next iteration's words formed between the steps (43.6), 16 steps an
+// iteration (39.4 there, but 13.3 -> 16.2 ms at dt 1e-3), 2 or 4 CTAs an SM.
 #include <type_traits>
 
 #include "walk_sched.cuh"

@@ -11,7 +11,8 @@
 // current item at once, and the warp opens the next item as soon as the
 // current one is fully handed out, however many earlier items still have
 // walks in flight.  Uneven exit times therefore idle no lane until the queue
-// is empty.
+// is empty; then, and in calls of few walks from the start, the lanes of a
+// warp share the walks that are left (cooperative rounds).
 //
 // Exit records.  A finished walk writes a small record (item, exit point,
 // hit fraction theta, wall, last material, per-material step counts) into a
@@ -19,8 +20,8 @@
 // warp turns them into samples g(exit) exp(-i (1/2) sum_m kappa_{e,m} T_m)
 // for every evaluation e, lane l handling evaluation l mod Epad.  The samples
 // of each item are summed across the lanes with warp shuffles (fixed order)
-// and lane e adds them to the item's slot in global memory (sum re, sum im,
-// sum re^2, sum im^2; a few MB, L2-resident).  An item belongs to the one
+// and added to the item's slot in global memory (sum re, sum im, sum re^2,
+// sum im^2; a few MB, L2-resident).  An item belongs to the one
 // warp that opened it, so its slot needs no atomics.  A second kernel adds
 // the slots of each node in item order.
 #pragma once
