@@ -721,9 +721,9 @@ def rbffd_measure(sdd, reps=2, cpu=True):
            "fp32_error": "the boundary walks are the main line's kernel and model: its fp32_error; "
                          "the RBF-FD stage is FP64",
            "roofline": {"bound": "latency",
-                        "note": "a BiCGStab iteration is 5 launches (replayed 8 iterations at a time as a "
-                                "CUDA graph) over vectors of 32k complex values (a few MB, L2-resident); the "
-                                "walks at the boundary nodes are bounded as the main line's kernel"}}
+                        "note": "all BiCGStab iterations run in one cooperative kernel (FP64 pipe, five grid "
+                                "barriers an iteration); the walks at the boundary nodes are bounded as the "
+                                "main line's kernel"}}
     if cpu:
         from oracle import rbffd as R
         sn, se_ = I.rect_grid(0, 0.9, 0, 0.9, 37, 37)
