@@ -153,8 +153,9 @@ struct WalkerF32 {
     // Shared address of the lane's column of WarpSmem::pend: the step that
     // ends a walk puts there the point before it, its proposed point, its
     // bridge uniform (negative: it overshot a wall) and its number.
-    // finalize() turns them into the exit record, for all ended lanes of the
-    // warp at once.  Through shared memory, not registers: the eight exits of
+    // They go into the warp's ring as they are, and finish() turns them into
+    // the exit record when 32 have gathered.  Through shared memory, not
+    // registers: the eight exits of
     // an unrolled iteration then leave nothing but the lane's state to merge
     // (in registers it cost 4.6 issue slots a step in moves).
     uint32_t pend;
@@ -346,7 +347,7 @@ struct WalkerF32 {
     // A warp takes this branch on about every second step (one lane of 32 is
     // enough), and the code stands once per unrolled step: it holds the
     // decision alone.  What follows a hit (the wall, theta, the exit point,
-    // the last material) waits for finalize().
+    // the last material) waits for finish().
     __device__ __forceinline__ static bool reaches_wall(const ModelDev &M, const WalkArgs &A, float X0,
                                                         float Z0, float Xn, float Zn, float dn, float pn,
                                                         uint32_t wa, uint32_t wb, float &U) {
@@ -360,15 +361,15 @@ struct WalkerF32 {
         return hit;
     }
 
-    // The exit record of an ended walk (st: 1 reached the boundary,
-    // 2 truncated).  Overshoot: theta_w = d_w / (d_w - d'_w) over the walls
+    // The exit record of an ended walk from what put_exit() left (tr: it was
+    // truncated).  Overshoot: theta_w = d_w / (d_w - d'_w) over the walls
     // with d'_w <= 0, smallest first, ties to the first of left, right, top,
     // bottom.  Bridge hit: the wall of the smallest product (first in wall
     // order) and theta = (2 d d' / dt) / (-ln U).
-    __device__ __forceinline__ void finalize(const ModelDev &M, const WalkArgs &A, int st, ExitInfo<float> &ei) const {
-        float X, Z, pXn, pZn, pU;
-        get_exit(X, Z, pXn, pZn, pU, ei.nocc);
-        if (st == 2) {
+    static constexpr bool kLate = true;
+    __device__ __forceinline__ static void finish(const ModelDev &M, const WalkArgs &A, int model, bool tr, float X,
+                                                  float Z, float pXn, float pZn, float pU, ExitInfo<float> &ei) {
+        if (tr) {
             ei.x = X; ei.z = Z; ei.th = 0.f; ei.wall = 0;
         } else {
             const float d[4] = {X + M.fhw, M.fhw - X, Z + M.fhh, M.fhh - Z};
@@ -392,7 +393,9 @@ struct WalkerF32 {
             }
             place(M, X, Z, pXn, pZn, best, bw, ei);
         }
-        ei.mlast = material(M, X, Z);
+        WalkerF32 t;
+        if (GC == GC_RASTER_MULTI) t.tco = A.models[model].tcoarse;
+        ei.mlast = t.material(M, X, Z);
     }
 
     // The part of an Euler step that does not depend on the position: the

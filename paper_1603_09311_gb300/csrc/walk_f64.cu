@@ -34,7 +34,7 @@ template <int KMAX_, int GEO>
 struct WalkerF64 {
     using Real = double;
     static constexpr int KMAX = KMAX_;
-    static constexpr bool kCoop = true, kAlone = false, kEvents = false, kTurns = false;  // every walk in cooperative rounds
+    static constexpr bool kCoop = true, kAlone = false, kEvents = false, kTurns = false, kLate = false;  // every walk in cooperative rounds
     static constexpr bool kGrouped = false;  // one queue (a grouped plan's order is one queue too)
     static constexpr int kMinCTAs = 2;       // the FP64 pipe is busy with 16 warps an SM
     using Occ = uint32_t;

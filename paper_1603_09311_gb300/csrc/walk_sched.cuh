@@ -142,7 +142,8 @@ __device__ __forceinline__ uint4 philox_rk(uint4 c, const uint32_t (&rk0)[10],
 template <class W>
 struct Ring {
     using Real = typename W::Real;
-    Real x[kRing], z[kRing], th[kRing];
+    Real x[kRing], z[kRing], th[kRing];  // W::kLate: the point before the exiting step and its
+    Real xn[W::kLate ? kRing : 1], zn[W::kLate ? kRing : 1];  // uniform, and its end, until the record is made
     uint32_t meta[kRing];  // wall | m_last << 2 | truncated << 6 | model << 8
     int32_t item[kRing];
     uint32_t n[kRing];     // occupation steps (all steps but the exiting one)
@@ -156,7 +157,7 @@ struct Ring {
 // the exit handler touches it.
 struct WarpState {
     unsigned long long steps[32];
-    unsigned long long walks, trunc;
+    unsigned long long trunc;
     double nx0, nz0;  // the current item's node,
     float fx0, fz0;   // and in single-precision centred coordinates
     int32_t disp_item, disp_rem, disp_model;
@@ -212,7 +213,8 @@ struct ExitInfo {
 //   start(M, A, S, path, model)  -- begin a walk at the warp's current node
 //   iterate(M, A, path, ExitInfo&) -> 0 running, 1 exited, 2 truncated
 //     (a few Euler steps per call; max_steps is a multiple of them)
-//   finalize(M, A, st, ExitInfo&): the exit record of a walk that has ended
+//   finalize(M, A, st, ExitInfo&): the exit record of a walk that has ended;
+//     kLate: get_exit() the exiting step instead, and finish() makes its record
 //   counts(M, nocc, c): steps spent in materials 1..KMAX-1 (at the exit,
 //     after nocc occupation steps)
 //   bind(h, p): the lane's columns of the occupancy histogram and of the
@@ -260,7 +262,7 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
     const bool dump = A.rec_steps != nullptr;
     S.steps[lane] = 0ull;
     if (lane == 0) {
-        S.walks = 0ull; S.trunc = 0ull;
+        S.trunc = 0ull;
         S.disp_item = -1; S.disp_rem = 0; S.disp_model = 0; S.disp_next = 0; S.nid = 0;
         S.head = S.tail = 0;
         S.queue_empty = 0;
@@ -367,7 +369,25 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
         const uint32_t head = S.head;
         const int Epad = M.Epad, my_e = lane & (Epad - 1);
         const int per_round = 32 / Epad, my_ro = lane / Epad;
-        const int rec_it = lane < cnt ? R.item[(head + lane) & (kRing - 1)] : -1;
+        const int mine_s = (head + lane) & (kRing - 1);
+        const int rec_it = lane < cnt ? R.item[mine_s] : -1;
+        if (lane < cnt) {
+            const uint32_t meta = R.meta[mine_s];
+            const bool tr = (meta >> 6) & 1u;
+            S.steps[lane] += (unsigned long long)R.n[mine_s] + (tr ? 0ull : 1ull);
+            if constexpr (W::kLate) {
+                // the exit records of all 32 at once (made by the few lanes of an
+                // exit batch they took 120 of its 350 instructions)
+                ExitInfo<Real> ex;
+                W::finish(M, A, (int)(meta >> 8), tr, R.x[mine_s], R.z[mine_s], R.xn[mine_s], R.zn[mine_s],
+                          R.th[mine_s], ex);
+                R.x[mine_s] = ex.x;
+                R.z[mine_s] = ex.z;
+                R.th[mine_s] = ex.th;
+                R.meta[mine_s] = meta | (uint32_t)ex.wall | ((uint32_t)ex.mlast << 2);
+            }
+        }
+        __syncwarp();
         unsigned pend = kFull >> (32 - cnt);
         while (pend) {
             const int it = __shfl_sync(kFull, rec_it, __ffs(pend) - 1);
@@ -503,30 +523,42 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
         const int nex = __popc(em);
         const uint32_t tail = S.tail;
         if (st != 0) {
-            w.finalize(M, A, st, ei);
             const int slot = (tail + __popc(em & lt_mask)) & (kRing - 1);
             const bool tr = st == 2;
-            R.x[slot] = ei.x;
-            R.z[slot] = ei.z;
-            R.th[slot] = ei.th;
-            R.meta[slot] = (uint32_t)ei.wall | ((uint32_t)ei.mlast << 2) | ((uint32_t)tr << 6) |
-                           ((uint32_t)model << 8);
+            uint32_t meta = ((uint32_t)tr << 6) | ((uint32_t)model << 8);
+            if constexpr (W::kLate) {
+                Real x0, z0, xn, zn, u;
+                w.get_exit(x0, z0, xn, zn, u, ei.nocc);
+                R.x[slot] = x0;
+                R.z[slot] = z0;
+                R.xn[slot] = xn;
+                R.zn[slot] = zn;
+                R.th[slot] = u;
+            } else {
+                w.finalize(M, A, st, ei);
+                R.x[slot] = ei.x;
+                R.z[slot] = ei.z;
+                R.th[slot] = ei.th;
+                meta |= (uint32_t)ei.wall | ((uint32_t)ei.mlast << 2);
+                R.aux[slot] = ei.aux;
+            }
+            R.meta[slot] = meta;
             R.item[slot] = item;
             R.n[slot] = ei.nocc;
-            R.path[slot] = path;
-            R.aux[slot] = ei.aux;
+            if (dump) {
+                R.path[slot] = path;
+                if constexpr (W::kLate) R.aux[slot] = 0;
+            }
             typename W::Occ c[W::kStored];
             w.counts(M, ei.nocc, c);
 #pragma unroll
             for (int j = 0; j < W::kStored; ++j) R.cnt[j][slot] = c[j];
-            S.steps[lane] += (unsigned long long)ei.nocc + (tr ? 0ull : 1ull);
             if (tr && !dump) atomicAdd(&A.item_trunc[item], 1);
         }
         const unsigned trm = __ballot_sync(kFull, st == 2);
         if (lane == 0) {
             S.tail = tail + (uint32_t)nex;
-            S.walks += (unsigned long long)nex;
-            S.trunc += (unsigned long long)__popc(trm);
+            if (trm) S.trunc += (unsigned long long)__popc(trm);
         }
         __syncwarp();
     };
@@ -622,7 +654,7 @@ __global__ void __launch_bounds__(256, W::kMinCTAs) walk_kernel(const __grid_con
     for (int off = 16; off > 0; off >>= 1) my_steps += __shfl_xor_sync(kFull, my_steps, off);
     if (lane == 0 && !dump) {
         atomicAdd(&A.counters[0], my_steps);
-        atomicAdd(&A.counters[1], S.walks);
+        atomicAdd(&A.counters[1], (unsigned long long)S.tail);  // every record was a walk
         atomicAdd(&A.counters[2], S.trunc);
     }
 }

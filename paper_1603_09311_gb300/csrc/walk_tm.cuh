@@ -41,7 +41,7 @@ struct WalkerTM {
     using Real = Real_;
     static constexpr int KMAX = KMAX_;
     static constexpr bool kF64 = sizeof(Real) == 8;
-    static constexpr bool kCoop = false, kAlone = true, kEvents = false, kTurns = false;
+    static constexpr bool kCoop = false, kAlone = true, kEvents = false, kTurns = false, kLate = false;
     using CoopInc = char;
     static constexpr bool kGrouped = false;
     static constexpr int kMinCTAs = 3;
@@ -386,7 +386,7 @@ template <int KMAX_>
 struct WalkerTM32 {
     using Real = float;
     static constexpr int KMAX = KMAX_;
-    static constexpr bool kCoop = true, kAlone = true, kEvents = true, kTurns = false;
+    static constexpr bool kCoop = true, kAlone = true, kEvents = true, kTurns = false, kLate = false;
     using CoopInc = float4;
     static constexpr bool kGrouped = false;
     static constexpr int kMinCTAs = 3;
