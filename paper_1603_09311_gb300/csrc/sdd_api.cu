@@ -836,13 +836,13 @@ WalkArgs base_args(sdd_ctx *ctx, const Launch &L, double dt, uint64_t seed) {
     A.max_steps = (uint32_t)L.max_steps;
     A.turns = phases_fit(ctx->M, dt);
     A.max_lanes = 32;
-    // Recording an ended walk and refilling its lane costs the warp about 300
+    // Recording an ended walk and refilling its lane costs the warp about 230
     // instructions, however many lanes take part; a lane that waits idles.
     // The best batch goes with the square root of the ended walks per step:
-    // measured optima at 150, 290, 970 steps a walk were 6, 4, 3 (dt 2e-3,
-    // 1e-3, 3e-4: 8.02 -> 6.92, 14.98 -> 14.07, 8.45 -> 8.18 ms against one at
-    // a time), none at 2900.  A walk takes about the domain's slowest decay
-    // time.
+    // measured optima at 150, 290, 970 steps a walk were 5, 4, 2 (dt 2e-3,
+    // 1e-3, 3e-4 on the quarter-space line: 13.36 -> 12.13, 11.05 -> 10.26,
+    // 28.8 -> 28.2 ms against one at a time), none at 2900.  A walk takes about
+    // the domain's slowest decay time.
     const double wx = 2.0 * ctx->M.hw, wz = 2.0 * ctx->M.hh;
     const double len = 2.0 / (9.8696 * (1.0 / (wx * wx) + 1.0 / (wz * wz))) / dt;
     A.exit_batch = (int32_t)std::min(6.0, std::max(1.0, std::floor(75.0 / std::sqrt(len) + 0.5)));

@@ -34,7 +34,7 @@ template <int KMAX_, int GEO>
 struct WalkerF64 {
     using Real = double;
     static constexpr int KMAX = KMAX_;
-    static constexpr bool kCoop = true, kAlone = false, kEvents = false, kTurns = false, kLate = false;  // every walk in cooperative rounds
+    static constexpr bool kCoop = true, kAlone = false, kEvents = false, kTurns = false;  // every walk in cooperative rounds
     static constexpr bool kGrouped = false;  // one queue (a grouped plan's order is one queue too)
     static constexpr int kMinCTAs = 2;       // the FP64 pipe is busy with 16 warps an SM
     using Occ = uint32_t;
@@ -172,13 +172,25 @@ struct WalkerF64 {
         p[160] = __hiloint2double(0, (int)k);
     }
 
-    // The exit record of an ended walk (st: 1 reached the boundary,
-    // 2 truncated), with the expressions of the definitions.
-    __device__ __forceinline__ void finalize(const ModelDev &M, const WalkArgs &A, int st, ExitInfo<double> &ei) const {
-        const double x0 = pend[0], z0 = pend[32], xn = pend[64], zn = pend[96], u = pend[128];
-        ei.nocc = (uint32_t)__double2loint(pend[160]);
+    // The exiting step as put_exit() left it.
+    __device__ __forceinline__ void get_exit(double &x0, double &z0, double &xn, double &zn, double &u,
+                                             uint32_t &k) const {
+        x0 = pend[0];
+        z0 = pend[32];
+        xn = pend[64];
+        zn = pend[96];
+        u = pend[128];
+        k = (uint32_t)__double2loint(pend[160]);
+    }
+
+    // The exit record of an ended walk (tr: it was truncated), with the
+    // expressions of the definitions.  For 32 walks at once: a walk alone held
+    // the FP64 pipe as long.
+    static constexpr bool kLate = true;
+    __device__ __forceinline__ static void finish(const ModelDev &M, const WalkArgs &A, int, bool tr, double x0,
+                                                  double z0, double xn, double zn, double u, ExitInfo<double> &ei) {
         ei.mlast = material(M, x0, z0);
-        if (st == 2) {
+        if (tr) {
             ei.x = x0; ei.z = z0; ei.th = 0.0; ei.wall = 0;
             return;
         }
