@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -292,7 +293,7 @@ __global__ void __launch_bounds__(kDotThreads) dot_partial_kernel(const Z *a, co
 }
 
 // Device-side BiCGStab scalars.  stop: 0 running, 1 converged, 2 breakdown,
-// 3 a barrier wait ran out.
+// 3 a barrier wait ran out, 4 the first one did (nothing was done).
 struct Scal {
     Z rho, alpha, omega, beta;
     double rnorm2, bnorm2, tol2;
@@ -516,8 +517,12 @@ __global__ void __launch_bounds__(kDotThreads / SPLIT, 2) bicgstab_kernel(const 
     };
     __syncthreads();
 
-    bool ok = true;
-    for (int it = 0; it < A.max_iter && !sh.stop; ++it) {
+    // all CTAs are on the GPU from here on: a wait for one that other kernels
+    // keep off it ends here, before anything is changed, and the host tries again
+    grid_arrive(A.bar, epoch);
+    bool ok = grid_wait(A.bar, epoch, &sh.bar_ok);
+    const bool came = ok;
+    for (int it = 0; ok && it < A.max_iter && !sh.stop; ++it) {
         const Z beta = sh.beta;
         for (int i = 0; i < nb; ++i) {
             const int row = KEEP ? row0 : row_of(i);
@@ -675,7 +680,7 @@ __global__ void __launch_bounds__(kDotThreads / SPLIT, 2) bicgstab_kernel(const 
         S.rho = sh.rho;
         S.rnorm2 = sh.rnorm2;
         S.iter = iter;
-        S.stop = ok ? sh.stop : 3;
+        S.stop = ok ? sh.stop : came ? 3 : 4;
         *A.S = S;
     }
 }
@@ -950,12 +955,22 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
     sa.nu = nu; sa.ns = ns;
     sa.blocks = (nu + kDotThreads - 1) / kDotThreads;
     const int kRun = 1024;
+    // One solve at a time: two cooperative grids that each wait for the rest of
+    // their CTAs would keep each other off the GPU.
+    static std::mutex solve_mu;
     for (int it = 0; it < max_iter && !h_S.stop;) {
+        std::lock_guard<std::mutex> lk(solve_mu);
         sa.max_iter = std::min(kRun, max_iter - it);
         RB_CUDA(cudaMemsetAsync(d_bar, 0, sizeof(unsigned), st));
         RB_CUDA(launch_bicgstab(sa, st));
         RB_CUDA(cudaMemcpyAsync(&h_S, d_S, sizeof(Scal), cudaMemcpyDeviceToHost, st));
         RB_CUDA(cudaStreamSynchronize(st));
+        if (h_S.stop == 4) {  // other kernels held the SMs for two seconds
+            h_S.stop = 0;
+            RB_CUDA(cudaMemcpyAsync(d_S, &h_S, sizeof(Scal), cudaMemcpyHostToDevice, st));
+            RB_CUDA(cudaStreamSynchronize(st));
+            continue;
+        }
         it += sa.max_iter;
     }
     if (h_S.stop == 3) return (sdd_status)report_error(SDD_E_CUDA, "a wait between the solver's blocks ran out");

@@ -60,3 +60,30 @@ def test_iteration_cap(max_iter):
     assert st["status"] == sdd.SDD_E_TIMEOUT and st["iterations"] <= max_iter
     if max_iter < 1024:
         assert st["iterations"] == max_iter
+
+
+def test_solves_beside_walks_and_in_several_threads():
+    # the solver's CTAs wait for one another: they must come through while
+    # walks fill the GPU on another stream, and with solves in other threads
+    import threading
+
+    cases = [_problem(60, 60, k) for k in range(3)]
+    alone = [sdd.sdd_rbffd_solve(*c, n_stencil=9, eps=5.0, tol=TOL)[0] for c in cases]
+    w = I.workload("quarterspace")
+    ctx = sdd.sdd_create(w["model"])
+    req = sdd.sdd_interface_values_async(ctx, w["nodes"], w["n_paths"] * 5, w["dt"], 3)
+    got = [None] * 3
+
+    def solve(k):
+        got[k] = sdd.sdd_rbffd_solve(*cases[k], n_stencil=9, eps=5.0, tol=TOL)[0]
+
+    threads = [threading.Thread(target=solve, args=(k,)) for k in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert req.wait() == sdd.SDD_OK
+    req.free()
+    ctx.close()
+    for a, b in zip(alone, got):
+        assert np.array_equal(a, b)
