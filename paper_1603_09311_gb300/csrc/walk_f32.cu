@@ -21,7 +21,7 @@
 //
 // What bounds it: instruction issue.  50 issue slots a step (64 nodes x 1e5
 // walks, dt 1e-4; 62 before the signs without flushing, one wall branch for
-// two steps and exits recorded apart) at 69 % of the issue rate, 5.4e11
+// two steps and exits recorded apart) at 69 % of the issue rate, 5.5e11
 // walk-steps/s; the rest of the rate goes to the wide multiplies of Philox
 // (dispatch and math-pipe stalls, with 2.4 of 6 warps eligible on average).
 // Tried without gain: region counters on the FMA pipe (40.2 -> 40.0 ms), the
