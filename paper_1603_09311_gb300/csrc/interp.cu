@@ -16,8 +16,9 @@
 //                         shared-memory scan, chunk prefixes)
 //   spline_factor_kernel  forward coefficients of the natural-spline
 //                         equations, one thread a row
-//   spline_cols_kernel    the spline's second derivatives of every unit knot
-//                         vector, one thread a column, as far as they matter
+//   spline_cols_kernel    G = the spline's second derivatives of every unit
+//                         knot vector, one thread a column, as far as they
+//                         matter
 //   linear_kernel, spline_kernel  values and standard errors
 //   scatter_kernel        the knots keep their own estimates
 #include <cmath>
@@ -82,8 +83,36 @@ __global__ void __launch_bounds__(kArcThreads) arc_kernel(int n, double *s) {
 // 12^-kWarm < 2^-64: every row is a thread's chain of kWarm divisions, not of
 // all rows before it (257 knots: 190 us -> 15 us).
 constexpr int kWarm = 18;
-__global__ void spline_factor_kernel(const double *s, int n, double *cp, double *rden) {
+
+// What the columns need to know of a call's data: the largest knot spacing (its
+// bits; of positive doubles these order as the doubles do), whether the weights
+// have to be kept whole, and the columns' farthest reach.
+struct SplineScan {
+    unsigned long long h_max;
+    int whole;   // a component of wide range, or not finite
+    int reach;   // largest |i - j| of a kept G[i][j]
+    double cut;  // entries of G below it are left out
+};
+
+// Columns keep the entries above 2^-100 / h_max^2: a weight is at most 0.13
+// h^2 max |G| besides its a or b, h the target's spacing, so what is left out
+// changes a weight by less than 2^-100, whatever the spacings.  (A cut against
+// the column's own largest entry is not enough: the weights carry h^2, and on
+// knots whose spacing grows by 2.6 or more a row they do not fall off at all.)
+// The weights add up to one, so where a component's largest modulus is at most
+// 2^40 times its smallest a sum loses less than 2^-60 a knot of the moduli of
+// its terms.  Other components (zeros, outliers, values that are not finite:
+// these count with any weight) keep every weight, and so do spacings whose
+// square leaves the double range.
+constexpr double kRange = 1099511627776.0;  // 2^40
+__device__ __forceinline__ double column_cut(const SplineScan &q) {
+    const double h = __longlong_as_double((long long)q.h_max), h2 = h * h;
+    return q.whole || !(h2 > 1e-290) || isinf(h2) ? 0.0 : 7.888609052210118e-31 / h2;
+}
+
+__global__ void spline_factor_kernel(const double *s, int n, double *cp, double *rden, SplineScan *scan) {
     const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row == 0) scan->cut = column_cut(*scan);
     if (row >= n - 2) return;
     double prev = 0.0, d = 0.0;
     for (int r = max(row - kWarm, 0); r <= row; ++r) {
@@ -97,74 +126,82 @@ __global__ void spline_factor_kernel(const double *s, int n, double *cp, double 
 }
 
 // Knot spacings must be positive (arc lengths of distinct nodes can still
-// round to equal sums): *err = 1 otherwise.
-__global__ void knots_check_kernel(const double *s, int n, int *err) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x + 1;
-    if (i < n && !(s[i] > s[i - 1])) atomicExch(err, 1);
-}
-
-// Column j of G: M(e_j), the second derivatives of the natural spline through
-// the unit vector e_j, kept by diagonals: G[i][j] at band[i (2 kBand + 1) + j -
-// i + kBand], |i - j| <= kBand, zero where not written.  The right-hand side
-// of row r (knot i = r + 1) is non-zero for i in {j - 1, j, j + 1} only, and
-// the entries fall off on both sides by at least 2/3 a row (0.27 on even
-// knots): a column ends where they are below 2^-100 of its largest, after
-// about 53 rows on even knots, at most after kBand, (2/3)^kBand < 2^-93.
-constexpr int kBand = 160;
-constexpr int kBandRow = 2 * kBand + 1;
-//
-// Every knot has a weight, however small, in every target's sum, so a value or
-// standard error that is not finite makes all of its component's results NaN;
-// the dropped weights must not hide one.  The CTAs past the columns (a warp
-// each, `from` on) look component c of v and of se through: spoil[c] is NaN if
-// it has one, else zero.
+// round to equal values).  scan (spline, else nullptr): the largest spacing; a
+// warp for each component of v and of se (from CTA `from` on) its range.
 __global__ void __launch_bounds__(32)
-    spline_cols_kernel(const double *s, int n, const double *cp, const double *rden, double *band, int from,
-                       const double *v, const double *se, int V, double *spoil) {
-    if ((int)blockIdx.x >= from) {
-        const int c = (int)blockIdx.x - from;
-        const double *u = c < V ? v + c : se + (c - V);
-        bool bad = false;
-        for (int j = threadIdx.x; j < n; j += 32) bad = bad || !isfinite(u[(size_t)j * V]);
-        const bool any = __any_sync(0xffffffffu, bad);
-        if (threadIdx.x == 0) spoil[c] = any ? nan("") : 0.0;
+    knots_check_kernel(const double *s, int n, int *err, int from, const double *v, const double *se, int V,
+                       SplineScan *scan) {
+    if ((int)blockIdx.x < from) {
+        const int i = blockIdx.x * 32 + threadIdx.x + 1;
+        if (i >= n) return;
+        const double h = s[i] - s[i - 1];
+        if (!(s[i] > s[i - 1])) atomicExch(err, 1);
+        else if (scan) atomicMax(&scan->h_max, (unsigned long long)__double_as_longlong(h));
         return;
     }
+    const int c = (int)blockIdx.x - from;
+    const double *u = c < V ? v + c : se + (c - V);
+    double big = 0.0, small = HUGE_VAL;
+    bool bad = false;
+    for (int j = threadIdx.x; j < n; j += 32) {
+        const double x = fabs(u[(size_t)j * V]);
+        bad = bad || !isfinite(x);
+        big = fmax(big, x);
+        small = fmin(small, x);
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+        big = fmax(big, __shfl_xor_sync(0xffffffffu, big, off));
+        small = fmin(small, __shfl_xor_sync(0xffffffffu, small, off));
+    }
+    bad = __any_sync(0xffffffffu, bad) || big > kRange * small;
+    if (bad && threadIdx.x == 0) scan->whole = 1;
+}
+
+// Column j of G [n][n]: M(e_j), the second derivatives of the natural spline
+// through the unit vector e_j; zero where not written.  The right-hand side of
+// row r (knot i = r + 1) is non-zero for i in {j - 1, j, j + 1} only, and the
+// entries fall off on both sides, by at least 2/3 a row (0.27 on even knots): a
+// column ends where they are below the cut, after about 53 rows on even knots.
+__global__ void __launch_bounds__(32)
+    spline_cols_kernel(const double *s, int n, const double *cp, const double *rden, double *G, SplineScan *scan) {
     const int j = blockIdx.x * 32 + threadIdx.x;
-    if (j >= n) return;
-    const int m = n - 2;
-    auto at = [&](int r) -> double & { return band[(size_t)(r + 1) * kBandRow + (j - r - 1 + kBand)]; };
-    const double tiny = 7.888609052210118e-31;  // 2^-100
-    const int r0 = max(j - 2, 0);               // first row with a right-hand side
-    const int rcap = min(m - 1, j - 1 + kBand);
-    double dprev = 0.0, big = 0.0;
-    int r1 = r0 - 1;
-    for (int r = r0; r <= rcap; ++r) {
-        const int i = r + 1;
-        const double hl = s[i] - s[i - 1];
-        double rhs = 0.0;
-        if (j >= i - 1 && j <= i + 1) {
-            const double hr = s[i + 1] - s[i];
-            if (j == i - 1) rhs = 6.0 / hl;
-            else if (j == i) rhs = -(6.0 / hl + 6.0 / hr);
-            else rhs = 6.0 / hr;
+    int reach = 0;
+    if (j < n) {
+        const int m = n - 2;
+        auto at = [&](int r) -> double & { return G[(size_t)(r + 1) * n + j]; };
+        const double cut = scan->cut;
+        const int r0 = max(j - 2, 0);  // first row with a right-hand side
+        double dprev = 0.0;
+        int r1 = r0 - 1;
+        for (int r = r0; r < m; ++r) {
+            const int i = r + 1;
+            const double hl = s[i] - s[i - 1];
+            double rhs = 0.0;
+            if (j >= i - 1 && j <= i + 1) {
+                const double hr = s[i + 1] - s[i];
+                if (j == i - 1) rhs = 6.0 / hl;
+                else if (j == i) rhs = -(6.0 / hl + 6.0 / hr);
+                else rhs = 6.0 / hr;
+            }
+            const double d = (rhs - hl * dprev) * rden[r];
+            at(r) = d;
+            dprev = d;
+            r1 = r;
+            if (r > j && fabs(d) < cut) break;
         }
-        const double d = (rhs - hl * dprev) * rden[r];
-        at(r) = d;
-        dprev = d;
-        r1 = r;
-        big = fmax(big, fabs(d));
-        if (r > j && fabs(d) < tiny * big) break;
+        double xnext = 0.0;
+        int low = r0;
+        for (int r = r1; r >= 0; --r) {
+            const double x = (r >= r0 ? at(r) : 0.0) - (r < m - 1 ? cp[r] * xnext : 0.0);
+            at(r) = x;
+            xnext = x;
+            low = r;
+            if (r < r0 && fabs(x) < cut) break;
+        }
+        reach = max(r1 + 1 - j, j - (low + 1));
     }
-    double xnext = 0.0;
-    const int rend = max(0, j - 1 - kBand);
-    for (int r = r1; r >= rend; --r) {
-        const double x = (r >= r0 ? at(r) : 0.0) - (r < m - 1 ? cp[r] * xnext : 0.0);
-        at(r) = x;
-        xnext = x;
-        big = fmax(big, fabs(x));
-        if (r < r0 && fabs(x) < tiny * big) break;
-    }
+    reach = __reduce_max_sync(0xffffffffu, reach);
+    if (threadIdx.x == 0) atomicMax(&scan->reach, reach);
 }
 
 // The target's segment: the largest i <= nk - 2 with s_i <= x.
@@ -204,71 +241,55 @@ __global__ void linear_kernel(const double *sk, int nk, const double *v, const d
 // CTA q: target q.  The weights
 //   c_j = a [j = i] + b [j = i + 1]
 //         + (a^3 - a) h^2 / 6 G[i][j] + (b^3 - b) h^2 / 6 G[i+1][j]
-// are formed once, a thread each, then every thread adds up components.  Zero
-// weights (beyond the columns' ends) are skipped.  With a thread for each
-// target and component and all knots in each sum, 1025 targets x 32
-// components x 257 knots took 0.35 ms; 0.05 ms so.
+// of the columns that reach the segment are formed once, a thread each, then
+// every thread adds up a component.  With a thread for each target and
+// component and all knots in each sum, 1025 targets x 32 components x 257 knots
+// took 0.35 ms.
 constexpr int kSplineThreads = 64;
-constexpr int kWeights = 2 * kBand + 2;
+constexpr int kWeights = 512;
 __global__ void __launch_bounds__(kSplineThreads)
-    spline_kernel(const double *sk, int nk, const double *band, const double *v, const double *se, int V,
-                  const double *spoil, const double *t, double *ov, double *ose) {
+    spline_kernel(const double *sk, int nk, const double *G, const SplineScan *scan, const double *v, const double *se,
+                  int V, const double *t, double *ov, double *ose) {
     __shared__ double w[kWeights];
-    __shared__ int16_t at[kWeights];
-    __shared__ int count;
     const size_t q = blockIdx.x;
     const double x = t[q];
     const int i = segment(sk, nk, x);
     const double h = sk[i + 1] - sk[i];
     const double a = (sk[i + 1] - x) / h, b = (x - sk[i]) / h;
     const double al = (a * a * a - a) * h * h / 6.0, be = (b * b * b - b) * h * h / 6.0;
-    const int j0 = max(i - kBand, 0), j1 = min(i + 1 + kBand, nk - 1);
-    for (int k = threadIdx.x; k <= j1 - j0; k += kSplineThreads) {
-        const int j = j0 + k, d = j - i;
-        double c = 0.0;
-        if (d <= kBand) c = al * band[(size_t)i * kBandRow + d + kBand];
-        if (d - 1 >= -kBand) c += be * band[(size_t)(i + 1) * kBandRow + d - 1 + kBand];
-        if (d == 0) c += a;
-        if (d == 1) c += b;
-        w[k] = c;
-    }
-    __syncthreads();
-    // the non-zero weights, in order
-    if (threadIdx.x < 32) {
-        int n = 0;
-        for (int k0 = 0; k0 <= j1 - j0; k0 += 32) {
-            const int k = k0 + threadIdx.x;
-            const double c = k <= j1 - j0 ? w[k] : 0.0;
-            const unsigned m = __ballot_sync(0xffffffffu, c != 0.0);
-            __syncwarp();
-            if (c != 0.0) {
-                const int o = n + __popc(m & ((1u << threadIdx.x) - 1u));
-                w[o] = c;
-                at[o] = (int16_t)k;
+    const double *gi = G + (size_t)i * nk, *gi1 = gi + nk;
+    const int reach = scan->whole ? nk : scan->reach;
+    const int j0 = max(i - reach, 0), j1 = min(i + 1 + reach, nk - 1);
+    for (int c0 = 0; c0 < V; c0 += kSplineThreads) {
+        const int c = c0 + threadIdx.x;
+        double val = 0.0, var = 0.0;
+        for (int k0 = j0; k0 <= j1; k0 += kWeights) {
+            const int n = min(j1 + 1 - k0, kWeights);
+            __syncthreads();
+            for (int k = threadIdx.x; k < n; k += kSplineThreads) {
+                const int j = k0 + k;
+                double cj = al * gi[j] + be * gi1[j];
+                if (j == i) cj += a;
+                if (j == i + 1) cj += b;
+                w[k] = cj;
             }
-            n += __popc(m);
-            __syncwarp();
-        }
-        if (threadIdx.x == 0) count = n;
-    }
-    __syncthreads();
-    const int n = count;
-    for (int c = threadIdx.x; c < V; c += kSplineThreads) {
-        double val = spoil[c], var = se ? spoil[V + c] : 0.0;
-        const double *vc = v + (size_t)j0 * V + c;
-        if (se) {
-            const double *ec = se + (size_t)j0 * V + c;
+            __syncthreads();
+            if (c >= V) continue;
+            const double *vc = v + (size_t)k0 * V + c;
+            if (se) {
+                const double *ec = se + (size_t)k0 * V + c;
 #pragma unroll 4
-            for (int k = 0; k < n; ++k) {
-                const size_t o = (size_t)at[k] * V;
-                val += w[k] * vc[o];
-                const double e = w[k] * ec[o];
-                var += e * e;
+                for (int k = 0; k < n; ++k) {
+                    val += w[k] * vc[(size_t)k * V];
+                    const double e = w[k] * ec[(size_t)k * V];
+                    var += e * e;
+                }
+            } else {
+#pragma unroll 4
+                for (int k = 0; k < n; ++k) val += w[k] * vc[(size_t)k * V];
             }
-        } else {
-#pragma unroll 4
-            for (int k = 0; k < n; ++k) val += w[k] * vc[(size_t)at[k] * V];
         }
+        if (c >= V) continue;
         ov[q * V + c] = val;
         if (ose) ose[q * V + c] = sqrt(var);
     }
@@ -324,28 +345,31 @@ sdd_status arg_error(const char *msg) { return (sdd_status)report_error(SDD_E_AR
 sdd_status run_interp(const double *d_sk, int nk, const double *d_v, const double *d_se, int V,
                       const double *d_t, int nt, int kind, double *d_ov, double *d_ose,
                       Scratch &S, cudaStream_t st, int *h_err) {
-    int *err;
-    INTERP_CUDA(S.alloc(&err, 1));
-    INTERP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
-    knots_check_kernel<<<(nk + 127) / 128, 128, 0, st>>>(d_sk, nk, err);
+    const bool spline = kind == SDD_INTERP_SPLINE && nk > 2;
+    struct Flags {
+        int err;
+        SplineScan scan;
+    } *flags;
+    INTERP_CUDA(S.alloc(&flags, 1));
+    INTERP_CUDA(cudaMemsetAsync(flags, 0, sizeof(Flags), st));
+    int *err = &flags->err;
+    SplineScan *scan = spline ? &flags->scan : nullptr;
+    const int pairs = (nk - 1 + 31) / 32, jobs = !spline ? 0 : d_se ? 2 * V : V;
+    knots_check_kernel<<<(unsigned)pairs + jobs, 32, 0, st>>>(d_sk, nk, err, pairs, d_v, d_se, V, scan);
     INTERP_CUDA(cudaGetLastError());
     const long long total = (long long)nt * V;
-    if (kind == SDD_INTERP_SPLINE && nk > 2) {
-        double *band, *cp, *rden, *spoil;
-        const int jobs = d_se ? 2 * V : V, cols = (nk + 31) / 32;
-        const size_t nband = (size_t)nk * kBandRow;
-        INTERP_CUDA(S.alloc(&band, nband));
+    if (spline) {
+        double *G, *cp, *rden;
+        INTERP_CUDA(S.alloc(&G, (size_t)nk * nk));
         INTERP_CUDA(S.alloc(&cp, (size_t)nk));
         INTERP_CUDA(S.alloc(&rden, (size_t)nk));
-        INTERP_CUDA(S.alloc(&spoil, (size_t)jobs));
-        INTERP_CUDA(cudaMemsetAsync(band, 0, nband * sizeof(double), st));
-        spline_factor_kernel<<<(nk + 63) / 64, 64, 0, st>>>(d_sk, nk, cp, rden);
+        INTERP_CUDA(cudaMemsetAsync(G, 0, (size_t)nk * nk * sizeof(double), st));
+        spline_factor_kernel<<<(nk + 63) / 64, 64, 0, st>>>(d_sk, nk, cp, rden, scan);
         INTERP_CUDA(cudaGetLastError());
-        spline_cols_kernel<<<cols + jobs, 32, 0, st>>>(d_sk, nk, cp, rden, band, cols, d_v, d_se, V, spoil);
+        spline_cols_kernel<<<(nk + 31) / 32, 32, 0, st>>>(d_sk, nk, cp, rden, G, scan);
         INTERP_CUDA(cudaGetLastError());
         if (total > 0) {
-            spline_kernel<<<(unsigned)nt, kSplineThreads, 0, st>>>(d_sk, nk, band, d_v, d_se, V, spoil, d_t, d_ov,
-                                                                   d_ose);
+            spline_kernel<<<(unsigned)nt, kSplineThreads, 0, st>>>(d_sk, nk, G, scan, d_v, d_se, V, d_t, d_ov, d_ose);
             INTERP_CUDA(cudaGetLastError());
         }
     } else if (total > 0) {
