@@ -341,8 +341,10 @@ constexpr long long kBarrierCycles = 4000000000ll;  // about two seconds
 constexpr unsigned kBarrierFail = 0x80000000u;
 
 // Barrier of all CTAs of the (cooperative) launch, in two halves.  A wait that
-// runs out sets the top bit of the counter; every CTA finds it at this wait or
-// its next one, and leaves.
+// runs out sets the top bit of the counter while arrivals are missing, by
+// compare-and-swap on the count it has just read: once all have arrived nobody
+// can fail the barrier any more, and until then nobody has passed it, so every
+// CTA leaves this barrier with the same answer.
 __device__ __forceinline__ void grid_arrive(unsigned *bar, unsigned &epoch) {
     epoch += gridDim.x;
     __syncthreads();
@@ -355,7 +357,10 @@ __device__ __forceinline__ bool grid_wait(unsigned *bar, unsigned epoch, int *ok
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
             if ((v & kBarrierFail) || v >= epoch) break;
-            if (clock64() - t0 > kBarrierCycles) v = atomicOr(bar, kBarrierFail) | kBarrierFail;
+            if (clock64() - t0 > kBarrierCycles && atomicCAS(bar, v, v | kBarrierFail) == v) {
+                v |= kBarrierFail;
+                break;
+            }
         }
         *ok = (v & kBarrierFail) == 0;
     }
