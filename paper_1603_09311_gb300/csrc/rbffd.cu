@@ -23,14 +23,17 @@
 //   assemble_kernel  one thread per unknown: the row (ELL, n slots, column
 //                    -1 for a Dirichlet neighbour), the diagonal and the
 //                    right-hand side
-//   bicgstab_kernel  all iterations in one cooperative launch (up to 1024 a
-//                    launch): element-wise updates, ELL matrix-vector
-//                    products and dot products between grid barriers
+//   bicgstab_kernel  the iterations, a few hundred in one cooperative launch:
+//                    element-wise updates, ELL matrix-vector products and dot
+//                    products between grid barriers
 #include <algorithm>
 #include <cmath>
+#include <condition_variable>
 #include <cstdint>
+#include <map>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -337,6 +340,7 @@ struct SolveArgs {
     int nu, ns, blocks, max_iter;
 };
 
+constexpr int kStaticSmem = 256;  // at least what the solver's kernel declares
 constexpr long long kBarrierCycles = 4000000000ll;  // about two seconds
 constexpr unsigned kBarrierFail = 0x80000000u;
 
@@ -469,11 +473,12 @@ __global__ void __launch_bounds__(kDotThreads / SPLIT, 2) bicgstab_kernel(const 
     Z(*sum)[T] = reinterpret_cast<Z(*)[T]>(solve_smem);                // [2 nbmax][T]
     double *sw = reinterpret_cast<double *>(sum + 2 * nbmax);          // KEEP: [ns][T]
     int32_t *sc = reinterpret_cast<int32_t *>(sw + (KEEP ? A.ns * T : 0));  // KEEP: [ns][T]
-    __shared__ struct {
+    __shared__ struct Shared {
         Z alpha, omega, beta, rho, aw;
         double rnorm2;
         int stop, bar_ok;
     } sh;
+    static_assert(sizeof(Shared) <= kStaticSmem, "static shared memory");
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     auto block_of = [&](int i) { return (int)blockIdx.x + i * stride; };
     auto row_of = [&](int i) { return (block_of(i) / SPLIT) * kDotThreads + t * SPLIT + block_of(i) % SPLIT; };
@@ -732,42 +737,126 @@ struct RbScratch {
     }
 };
 
+// A launch of the solver's kernel: its grid, and how many of its CTAs an SM
+// takes.
+struct SolveLaunch {
+    const void *kernel = nullptr;
+    int ctas = 0, per = 0, threads = 0;
+    size_t smem = 0;
+};
+
+// Iterations of a turn, which another solve waits for at most, and of a launch.
+// A turn ends with the host waiting for it (80 us).  A grid of more CTAs than
+// SMs leaves no registers for other kernels, so its turns are short and cut
+// into short launches, between which those get in.  Two solves of 300 x 300
+// nodes (70 ms alone) from two threads: 102 ms so, 115 with 64 iterations a
+// launch and 256 a turn, 125 with 256 and 256, 137 one after the other; alone
+// the same within 1 %.
+constexpr int kTurn = 1024, kFullTurn = 128, kFullRun = 32;
+
+// At most ctas_max CTAs.  KEEP: *L stays empty where the blocks are more.
 template <int SPLIT, bool KEEP>
-cudaError_t launch_solve(const SolveArgs &A, int n_sm, bool *fits, cudaStream_t st) {
+cudaError_t shape_solve(const SolveArgs &A, int n_sm, int ctas_max, SolveLaunch *L) {
     constexpr int T = kDotThreads / SPLIT;
-    // KEEP: one block a CTA; else at most eight (1024 blocks, two CTAs on each
-    // of at least 64 SMs)
     const int parts = A.blocks * SPLIT;
-    const int nb = KEEP ? 1 : (parts + 2 * n_sm - 1) / (2 * n_sm);
-    const size_t smem = (size_t)nb * 2 * T * sizeof(Z) +
-                        (KEEP ? (size_t)A.ns * T * (sizeof(double) + sizeof(int32_t)) : 0);
     auto k = bicgstab_kernel<SPLIT, KEEP>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, T, smem);
-    if (e != cudaSuccess) return e;
-    *fits = parts <= per * n_sm;
-    if (KEEP && !*fits) return cudaSuccess;
-    if (!KEEP && (long long)per * n_sm * nb < parts) return cudaErrorLaunchOutOfResources;
-    SolveArgs a = A;
-    void *args[] = {&a};
-    return cudaLaunchCooperativeKernel((const void *)k, dim3(std::min(parts, per * n_sm)), dim3(T), args, smem, st);
+    // the same attributes for every solve: others may be launching in other threads
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - kStaticSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    while (e == cudaSuccess && ctas_max > 0 && (!KEEP || parts <= ctas_max)) {
+        const int ctas = std::min(parts, ctas_max), nb = (parts + ctas - 1) / ctas;
+        const size_t smem = (size_t)nb * 2 * T * sizeof(Z) +
+                            (KEEP ? (size_t)A.ns * T * (sizeof(double) + sizeof(int32_t)) : 0);
+        int per = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, T, smem);
+        if (e != cudaSuccess) return e;
+        if (ctas <= per * n_sm) {
+            *L = SolveLaunch{(const void *)k, ctas, per, T, smem};
+            return cudaSuccess;
+        }
+        ctas_max = per * n_sm;
+    }
+    return e != cudaSuccess || KEEP ? e : cudaErrorLaunchOutOfResources;
 }
 
 // Two CTAs a block of rows while that leaves at most one CTA an SM (FP64 time
-// halves, see bicgstab_kernel); one with the row in registers while all blocks
-// are resident; else several blocks a CTA.
-cudaError_t launch_bicgstab(const SolveArgs &A, cudaStream_t st) {
-    int dev = 0, n_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    bool fits = false;
-    if (2 * A.blocks <= n_sm) return launch_solve<2, true>(A, n_sm, &fits, st);
-    e = launch_solve<1, true>(A, n_sm, &fits, st);
-    if (e != cudaSuccess || fits) return e;
-    return launch_solve<1, false>(A, n_sm, &fits, st);
+// halves, see bicgstab_kernel); one with the row in registers up to ctas_max
+// blocks; else several blocks a CTA.
+cudaError_t shape_bicgstab(const SolveArgs &A, int n_sm, int ctas_max, SolveLaunch *L) {
+    *L = SolveLaunch{};
+    if (2 * A.blocks <= n_sm) return shape_solve<2, true>(A, n_sm, ctas_max, L);
+    cudaError_t e = shape_solve<1, true>(A, n_sm, ctas_max, L);
+    if (e != cudaSuccess || L->kernel) return e;
+    return shape_solve<1, false>(A, n_sm, ctas_max, L);
 }
+
+// Solves in flight on one device.  The CTAs of a grid wait for one another, so
+// all grids in flight must fit on the GPU together.  With p the smallest number
+// of CTAs an SM takes of any of their kernels, no CTA needs more than 1 / p of
+// an SM: an SM that cannot take one more has p, and grids of together at most
+// p x SMs CTAs all come through.  Launches go in the order of their tickets.
+struct SolverQueue {
+    std::mutex mu;
+    std::condition_variable cv;
+    uint64_t next = 0, serving = 0;
+    int solves = 0;                             // solves between their first launch and their last
+    std::vector<std::pair<int, int>> in_flight; // (CTAs, CTAs an SM takes)
+
+    bool fits(const SolveLaunch &L, int n_sm) const {
+        long long sum = L.ctas;
+        int p = L.per;
+        for (const auto &f : in_flight) {
+            sum += f.first;
+            p = std::min(p, f.second);
+        }
+        return in_flight.empty() || sum <= (long long)p * n_sm;
+    }
+};
+
+SolverQueue &solver_queue(int dev) {
+    static std::mutex mu;
+    static std::map<int, SolverQueue> queues;
+    std::lock_guard<std::mutex> lk(mu);
+    return queues[dev];
+}
+
+// A solve's place among those of its device, from its first launch to its last.
+struct SolverSeat {
+    SolverQueue &Q;
+    explicit SolverSeat(SolverQueue &q) : Q(q) {
+        std::lock_guard<std::mutex> lk(Q.mu);
+        ++Q.solves;
+    }
+    ~SolverSeat() {
+        std::lock_guard<std::mutex> lk(Q.mu);
+        --Q.solves;
+    }
+    // Waits for this launch's turn and for room.  alone, shared: the grid of a
+    // solve that has the GPU to itself, and of one among others.
+    SolveLaunch enter(const SolveLaunch &alone, const SolveLaunch &shared, int n_sm) {
+        std::unique_lock<std::mutex> lk(Q.mu);
+        const uint64_t me = Q.next++;
+        SolveLaunch L;
+        Q.cv.wait(lk, [&] {
+            L = Q.solves > 1 ? shared : alone;
+            return Q.serving == me && Q.fits(L, n_sm);
+        });
+        Q.in_flight.emplace_back(L.ctas, L.per);
+        ++Q.serving;
+        Q.cv.notify_all();
+        return L;
+    }
+    void leave(const SolveLaunch &L) {
+        std::lock_guard<std::mutex> lk(Q.mu);
+        Q.in_flight.erase(std::find(Q.in_flight.begin(), Q.in_flight.end(), std::make_pair(L.ctas, L.per)));
+        Q.cv.notify_all();
+    }
+};
 
 sdd_status check_nodes_eps(const double *nodes_xz, int32_t n, int32_t ns, double eps) {
     if (ns < 2 || ns > kMaxStencil) return rb_arg("n_stencil must be in 2 .. SDD_RBFFD_MAX_STENCIL");
@@ -952,31 +1041,56 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
     RB_CUDA(cudaMemcpyAsync(d_S, &h_S, sizeof(Scal), cudaMemcpyHostToDevice, st));
     RB_CUDA(cudaEventRecord(S.ev[3], st));
 
-    // iterations, up to kRun in one cooperative launch
+    // iterations
     SolveArgs sa{};
     sa.ew = d_ew; sa.ecol = d_ecol; sa.unk = d_unk; sa.kappa = d_kap; sa.dinv = d_dinv; sa.rh = rh;
     sa.r = rr; sa.p = p; sa.v = v; sa.x = x; sa.y = y; sa.z = zz; sa.s = s; sa.t = t;
     sa.part = d_part; sa.S = d_S; sa.bar = d_bar;
     sa.nu = nu; sa.ns = ns;
     sa.blocks = (nu + kDotThreads - 1) / kDotThreads;
-    const int kRun = 1024;
-    // One solve at a time: two cooperative grids that each wait for the rest of
-    // their CTAs would keep each other off the GPU.
-    static std::mutex solve_mu;
-    for (int it = 0; it < max_iter && !h_S.stop;) {
-        std::lock_guard<std::mutex> lk(solve_mu);
-        sa.max_iter = std::min(kRun, max_iter - it);
-        RB_CUDA(cudaMemsetAsync(d_bar, 0, sizeof(unsigned), st));
-        RB_CUDA(launch_bicgstab(sa, st));
-        RB_CUDA(cudaMemcpyAsync(&h_S, d_S, sizeof(Scal), cudaMemcpyDeviceToHost, st));
-        RB_CUDA(cudaStreamSynchronize(st));
-        if (h_S.stop == 4) {  // other kernels held the SMs for two seconds
-            h_S.stop = 0;
-            RB_CUDA(cudaMemcpyAsync(d_S, &h_S, sizeof(Scal), cudaMemcpyHostToDevice, st));
-            RB_CUDA(cudaStreamSynchronize(st));
-            continue;
+    int dev = 0, n_sm = 0;
+    RB_CUDA(cudaGetDevice(&dev));
+    RB_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+    // alone: all the CTAs that fit; beside other solves: half of them
+    SolveLaunch alone, shared;
+    RB_CUDA(shape_bicgstab(sa, n_sm, 2 * n_sm, &alone));
+    if (alone.ctas > n_sm) RB_CUDA(shape_bicgstab(sa, n_sm, n_sm, &shared));
+    else shared = alone;
+    {
+        SolverSeat seat(solver_queue(dev));
+        int it = 0;
+        // one turn: *done iterations, if it does not stop
+        auto turn = [&](int *done) -> cudaError_t {
+            const SolveLaunch L = seat.enter(alone, shared, n_sm);
+            const bool full = L.ctas > n_sm;
+            const int end = std::min(max_iter - it, full ? kFullTurn : kTurn);
+            cudaError_t e = cudaSuccess;
+            for (*done = 0; *done < end && e == cudaSuccess; *done += sa.max_iter) {
+                sa.max_iter = std::min(end - *done, full ? kFullRun : kTurn);
+                void *args[] = {&sa};
+                e = cudaMemsetAsync(d_bar, 0, sizeof(unsigned), st);
+                if (e == cudaSuccess)
+                    e = cudaLaunchCooperativeKernel(L.kernel, dim3(L.ctas), dim3(L.threads), args, L.smem, st);
+            }
+            // waited for before the copy: a copy to pageable memory waits for the
+            // grid inside the driver, and other threads' copies wait with it
+            const cudaError_t es = cudaStreamSynchronize(st);
+            seat.leave(L);
+            if (e == cudaSuccess) e = es;
+            if (e == cudaSuccess) e = cudaMemcpyAsync(&h_S, d_S, sizeof(Scal), cudaMemcpyDeviceToHost, st);
+            return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+        };
+        while (it < max_iter && !h_S.stop) {
+            int done = 0;
+            RB_CUDA(turn(&done));
+            if (h_S.stop == 4) {  // other kernels held the SMs for two seconds
+                h_S.stop = 0;
+                RB_CUDA(cudaMemcpyAsync(d_S, &h_S, sizeof(Scal), cudaMemcpyHostToDevice, st));
+                RB_CUDA(cudaStreamSynchronize(st));
+                continue;
+            }
+            it += done;
         }
-        it += sa.max_iter;
     }
     if (h_S.stop == 3) return (sdd_status)report_error(SDD_E_CUDA, "a wait between the solver's blocks ran out");
     // the true residual |b - K x| / |b|
