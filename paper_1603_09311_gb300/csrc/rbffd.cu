@@ -343,6 +343,9 @@ struct SolveArgs {
 constexpr int kStaticSmem = 256;  // at least what the solver's kernel declares
 constexpr long long kBarrierCycles = 4000000000ll;  // about two seconds
 constexpr unsigned kBarrierFail = 0x80000000u;
+// Launches in a row whose CTAs did not all get onto the GPU (ten minutes)
+// before a solve gives up.
+constexpr int kTries = 300;
 
 // Barrier of all CTAs of the (cooperative) launch, in two halves.  A wait that
 // runs out sets the top bit of the counter while arrivals are missing, by
@@ -1058,15 +1061,14 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
     else shared = alone;
     {
         SolverSeat seat(solver_queue(dev));
-        int it = 0;
-        // one turn: *done iterations, if it does not stop
-        auto turn = [&](int *done) -> cudaError_t {
+        int tries = 0;
+        auto turn = [&]() -> cudaError_t {
             const SolveLaunch L = seat.enter(alone, shared, n_sm);
             const bool full = L.ctas > n_sm;
-            const int end = std::min(max_iter - it, full ? kFullTurn : kTurn);
+            int left = std::min(max_iter - h_S.iter, full ? kFullTurn : kTurn);
             cudaError_t e = cudaSuccess;
-            for (*done = 0; *done < end && e == cudaSuccess; *done += sa.max_iter) {
-                sa.max_iter = std::min(end - *done, full ? kFullRun : kTurn);
+            for (; left > 0 && e == cudaSuccess; left -= sa.max_iter) {
+                sa.max_iter = std::min(left, full ? kFullRun : kTurn);
                 void *args[] = {&sa};
                 e = cudaMemsetAsync(d_bar, 0, sizeof(unsigned), st);
                 if (e == cudaSuccess)
@@ -1080,16 +1082,17 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
             if (e == cudaSuccess) e = cudaMemcpyAsync(&h_S, d_S, sizeof(Scal), cudaMemcpyDeviceToHost, st);
             return e != cudaSuccess ? e : cudaStreamSynchronize(st);
         };
-        while (it < max_iter && !h_S.stop) {
-            int done = 0;
-            RB_CUDA(turn(&done));
+        while (h_S.iter < max_iter && !h_S.stop) {
+            RB_CUDA(turn());
             if (h_S.stop == 4) {  // other kernels held the SMs for two seconds
+                if (++tries == kTries)
+                    return (sdd_status)report_error(SDD_E_CUDA, "other kernels kept the solver's blocks off the GPU");
                 h_S.stop = 0;
                 RB_CUDA(cudaMemcpyAsync(d_S, &h_S, sizeof(Scal), cudaMemcpyHostToDevice, st));
                 RB_CUDA(cudaStreamSynchronize(st));
                 continue;
             }
-            it += done;
+            tries = 0;
         }
     }
     if (h_S.stop == 3) return (sdd_status)report_error(SDD_E_CUDA, "a wait between the solver's blocks ran out");
