@@ -17,6 +17,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "../../include/sdd.h"
 #include "sdd_internal.cuh"
 
@@ -969,16 +971,33 @@ sdd_status run(sdd_ctx *ctx, const Plan &P, const Launch &L, WalkArgs A, cudaStr
 
 }  // namespace
 
+namespace {
+// The current context's id, which no other context of the process ever has: a
+// device that other code has reset comes back with another one.
+cudaError_t context_id(unsigned long long *id) {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q);
+    if (e != cudaSuccess) return e;
+    if (q != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
+    return reinterpret_cast<CUresult (*)(CUcontext, unsigned long long *)>(f)(nullptr, id) == CUDA_SUCCESS
+               ? cudaSuccess
+               : cudaErrorDeviceUninitialized;
+}
+}  // namespace
+
 cudaError_t sdd::scratch_alloc(void **p, size_t bytes, cudaStream_t st) {
     static std::mutex mu;
-    static std::map<int, cudaMemPool_t> pools;  // one a device, for the life of the process
+    static std::map<unsigned long long, cudaMemPool_t> pools;  // one a context; a pool ends with its context
     int dev = 0;
+    unsigned long long ctx = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = context_id(&ctx);
     if (e != cudaSuccess) return e;
     cudaMemPool_t pool = nullptr;
     {
         std::lock_guard<std::mutex> lk(mu);
-        auto it = pools.find(dev);
+        auto it = pools.find(ctx);
         if (it == pools.end()) {
             cudaMemPoolProps props{};
             props.allocType = cudaMemAllocationTypePinned;
@@ -992,7 +1011,7 @@ cudaError_t sdd::scratch_alloc(void **p, size_t bytes, cudaStream_t st) {
                 cudaMemPoolDestroy(pool);
                 return e;
             }
-            pools[dev] = pool;
+            pools[ctx] = pool;
         } else {
             pool = it->second;
         }

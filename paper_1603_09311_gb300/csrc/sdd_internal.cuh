@@ -250,11 +250,11 @@ cudaError_t launch_walk_f64(int kmax, int geo, const ModelDev &M, const WalkArgs
 int report_error(int status, const char *msg);
 
 // Device scratch of one call on its stream (interpolation, resistivity,
-// RBF-FD), from a pool of the library's own on the current device: an
+// RBF-FD), from a pool of the library's own in the current context: an
 // allocation and its release are stream-ordered and safe from several threads,
 // and between calls the pool keeps at most kScratchKeep bytes, the rest goes
-// back to the device.  cudaMalloc and cudaFree for each array took 1.3 ms of a
-// 16.6 ms sub-domain solve (25 arrays) and 0.2 ms of a 0.4 ms interpolation.
+// back to the device.  cudaMalloc and cudaFree for each array took 0.7 ms of a
+// 17.7 ms sub-domain solve (25 arrays) and 0.15 ms of a 0.42 ms interpolation.
 constexpr uint64_t kScratchKeep = 64ull << 20;
 cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st);
 
