@@ -2229,7 +2229,6 @@ extern "C" sdd_status sdd_batch_values(const sdd_batch_entry *entries, int32_t n
     A.nodes = (const double *)own->nodes.p;
     A.node_ids = (const uint32_t *)own->node_ids.p;
     A.models = (const BatchModel *)own->batch_models.p;
-    A.turns = std::all_of(table.begin(), table.end(), [](const BatchModel &B) { return B.turns != 0; });
     st = run(own, P, L, A, s, true, true, (double *)own->mean.p, (double *)own->se.p, n_nodes, &Mb);
     if (st != SDD_OK) return st;
     std::vector<double> hm(ob / sizeof(double)), hs(ob / sizeof(double));
@@ -2497,7 +2496,6 @@ sdd_status srv_launch(sdd_server *srv, SrvLane &L, std::vector<SrvPiece> &batch)
     A.queue = (int32_t *)L.queue.p;
     A.error = (int32_t *)L.err.p;
     A.models = (const BatchModel *)L.models.p;
-    A.turns = std::all_of(table.begin(), table.end(), [](const BatchModel &B) { return B.turns != 0; });
     ModelDev Mb = srv->tmpl->M;
     Mb.gcode = GC_RASTER_MULTI;
     Mb.K = Kmax;

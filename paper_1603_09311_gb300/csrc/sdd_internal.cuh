@@ -206,7 +206,7 @@ struct WalkArgs {
     uint32_t key0, key1;       // Philox key (seed)
     uint32_t rk0[10], rk1[10]; // the key of each Philox round (key bumped by the Weyl constants)
     uint32_t max_steps;
-    int32_t turns;             // single precision: every kappa dt / (4 pi) is below kMaxTurns
+    int32_t turns;             // single precision: every kappa dt / (4 pi) is below kMaxTurns (batched: BatchModel)
     int32_t exit_batch;        // ended walks of a warp recorded together (1 .. 32)
     int32_t max_lanes;         // walks of a warp at a time (1 .. 32)
     double *slots;             // [n_items][E][4]: sum re, sum im, sum re^2, sum im^2

@@ -636,7 +636,9 @@ struct WalkerF32 {
         const bool multi = GC == GC_RASTER_MULTI;
         const int K = multi ? A.models[model].K : M.K;
         float pr;
-        if (A.turns) {
+        // a batched model's own flag: its samples are those it has alone,
+        // whatever the launch's other models are
+        if (multi ? A.models[model].turns : A.turns) {
             const uint64_t *f = (multi ? A.models[model].turn_frac : T.turn_frac) + e * K;
             const uint32_t whole = (multi ? A.models[model].turn_whole : T.turn_whole)[e * K + mlast];
             uint64_t turn = 0;
