@@ -797,12 +797,15 @@ bool phases_fit(const ModelDev &M, double dt) {
     return true;
 }
 
-// The sample constants of a model of a batched launch.
+// The rates and boundary constants of a model of a batched launch.
 void fill_samples(BatchModel &B, const ModelDev &M, double dt) {
     for (int k = 0; k < M.E; ++k) B.ev[k] = eval_f(M.ev[k]);
     B.turns = phases_fit(M, dt);
-    if (!B.turns) return;
     for (int k = 0; k < M.E * M.K; ++k) {
+        if (!B.turns) {
+            B.kappa[k] = M.kappa[k];
+            continue;
+        }
         const PhaseTurn p = phase_turn(M.kappa[k], dt);
         B.turn_frac[k] = p.frac;
         B.turn_whole[k] = p.whole;
@@ -2208,7 +2211,6 @@ extern "C" sdd_status sdd_batch_values(const sdd_batch_entry *entries, int32_t n
         B.tcoarse = c->M.tcoarse;
         B.tpool = c->M.tpool;
         B.K = c->K;
-        for (int k = 0; k < c->E * c->K; ++k) B.kappa[k] = c->M.kappa[k];
         fill_samples(B, c->M, dt);
     }
     cudaStream_t s = own->stream;
@@ -2352,10 +2354,10 @@ struct sdd_server {
 
 namespace {
 
-// What a request is charged for its rates and boundary constants (the phase
-// tables made from them for a launch are not charged).
-constexpr int64_t kModelCharge = sizeof(BatchModel) - sizeof(BatchModel::turn_frac) - sizeof(BatchModel::turn_whole) +
-                                 kMaxE * (sizeof(EvalDev) - sizeof(EvalF));
+// What a request is charged for its model in a launch's table: its rates, its
+// boundary constants in double precision and its tile map's addresses.
+constexpr int64_t kModelCharge = kMaxE * kMaxK * sizeof(double) + kMaxE * sizeof(EvalDev) + 32;
+static_assert((int64_t)sizeof(BatchModel) <= kModelCharge, "a model's table entry exceeds what its request is charged");
 
 int64_t request_bytes(const sdd_server *srv, int32_t n_nodes) {
     const int E = srv->cfg.n_eval;
@@ -2800,7 +2802,6 @@ extern "C" sdd_status sdd_server_submit(sdd_server *srv, const sdd_request_desc 
     std::memset(&r->bm, 0, sizeof(r->bm));
     r->K = m->n_materials;
     r->bm.K = m->n_materials;
-    for (int k = 0; k < md.E * md.K; ++k) r->bm.kappa[k] = md.kappa[k];
     fill_samples(r->bm, md, srv->cfg.dt);
     const int n = req->n_nodes, E = c.n_eval;
     r->nodes.assign(req->nodes_xz, req->nodes_xz + 2 * n);

@@ -142,11 +142,13 @@ struct BatchModel {
     const int8_t *raster;
     const uint32_t *tcoarse;
     const uint8_t *tpool;
-    int32_t K, turns;             // turns: the phases fit PhaseTurn
-    double kappa[kMaxE * kMaxK];  // [E][K] of this model
-    EvalF ev[kMaxE];
-    uint64_t turn_frac[kMaxE * kMaxK];   // PhaseTurn of each kappa at the launch's dt
+    int32_t K, turns;                       // turns: the phases fit PhaseTurn
+    union {
+        double kappa[kMaxE * kMaxK];        // [E][K] of this model; turns:
+        uint64_t turn_frac[kMaxE * kMaxK];  // PhaseTurn of each kappa at the launch's dt
+    };
     uint32_t turn_whole[kMaxE * kMaxK];
+    EvalF ev[kMaxE];
 };
 
 struct ModelDev {
