@@ -846,8 +846,16 @@ WalkArgs base_args(sdd_ctx *ctx, const Launch &L, double dt, uint64_t seed) {
     // The best batch goes with the square root of the ended walks per step:
     // measured optima at 150, 290, 970 steps a walk were 5, 4, 2 (dt 2e-3,
     // 1e-3, 3e-4 on the quarter-space line: 13.36 -> 12.13, 11.05 -> 10.26,
-    // 28.8 -> 28.2 ms against one at a time), none at 2900.  A walk takes about
-    // the domain's slowest decay time.
+    // 28.8 -> 28.2 ms against one at a time), none at 2900.  A TE walk takes
+    // about the domain's slowest decay time.  TM walks are recorded one at a
+    // time: their lengths go with the strips' diffusions, and waiting lanes cost
+    // more (FP64, 256 nodes x 4000 walks, dt 1e-3 and 2e-3: 126 -> 124 and 69 ->
+    // 67 ms against this rule's batches of 4 and 5; FP32, diffusions 0.05 and
+    // 0.1: 45.9 -> 44.7 ms; 1 and 10: the same).
+    if (ctx->geo == GEO_TM) {
+        A.exit_batch = 1;
+        return A;
+    }
     const double wx = 2.0 * ctx->M.hw, wz = 2.0 * ctx->M.hh;
     const double len = 2.0 / (9.8696 * (1.0 / (wx * wx) + 1.0 / (wz * wz))) / dt;
     A.exit_batch = (int32_t)std::min(6.0, std::max(1.0, std::floor(75.0 / std::sqrt(len) + 0.5)));
