@@ -721,7 +721,7 @@ def rbffd_measure(sdd, reps=2, cpu=True):
            "fp32_error": "the boundary walks are the main line's kernel and model: its fp32_error; "
                          "the RBF-FD stage is FP64",
            "roofline": {"bound": "latency",
-                        "note": "all BiCGStab iterations run in one cooperative kernel (FP64 pipe, five grid "
+                        "note": "the BiCGStab iterations run in cooperative launches (FP64 pipe, five grid "
                                 "barriers an iteration); the walks at the boundary nodes are bounded as the "
                                 "main line's kernel"}}
     if cpu:

@@ -589,7 +589,7 @@ sdd_status sdd_apparent_from_values(const double *values, const double *se, int3
  *    by BiCGStab with a Jacobi preconditioner to |b - K x| <= tol |b|.
  * The paper uses n_stencil = 9 and eps = 1/2000 per metre with 100-125 m
  * spacing (eps h about 0.05).  FP64 on the current device; host arrays. */
-#define SDD_RBFFD_MAX_NODES (1 << 18) /* the neighbour search scans all nodes */
+#define SDD_RBFFD_MAX_NODES (1 << 18)
 #define SDD_RBFFD_MAX_STENCIL 16
 
 typedef struct {
@@ -598,7 +598,7 @@ typedef struct {
     double rel_residual;  /* |b - K x| / |b| of the returned solution */
     double knn_ms;        /* device time of the neighbour search */
     double weights_ms;    /* device time of the weights */
-    double solve_ms;      /* device time of assembly and BiCGStab (with its polls) */
+    double solve_ms;      /* device time of assembly and BiCGStab, waits beside other solves included */
 } sdd_rbffd_stats;
 
 /* Stencils and Laplacian weights of every node.

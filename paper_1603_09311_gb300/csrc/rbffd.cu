@@ -270,29 +270,19 @@ __global__ void spmv_kernel(const double *ew, const int32_t *ecol, int nu, int n
     y[r] = acc;
 }
 
-// Block partials of sum conj(a_i) b_i (and of sum conj(a_i) c_i when c).
-__global__ void __launch_bounds__(kDotThreads) dot_partial_kernel(const Z *a, const Z *b, const Z *c,
-                                                                  int n, Z *part_b, Z *part_c) {
-    __shared__ Z sb[kDotThreads], sc[kDotThreads];
-    Z ab = {0.0, 0.0}, ac = {0.0, 0.0};
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        ab = zadd(ab, zcdot(a[i], b[i]));
-        if (c) ac = zadd(ac, zcdot(a[i], c[i]));
-    }
-    sb[threadIdx.x] = ab;
-    sc[threadIdx.x] = ac;
+// Block partials of |a|^2, in the real part.
+__global__ void __launch_bounds__(kDotThreads) norm_partial_kernel(const Z *a, int n, Z *part) {
+    __shared__ Z sum[kDotThreads];
+    Z acc = {0.0, 0.0};
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        acc = zadd(acc, zcdot(a[i], a[i]));
+    sum[threadIdx.x] = acc;
     __syncthreads();
     for (int off = kDotThreads / 2; off > 0; off >>= 1) {
-        if (threadIdx.x < off) {
-            sb[threadIdx.x] = zadd(sb[threadIdx.x], sb[threadIdx.x + off]);
-            sc[threadIdx.x] = zadd(sc[threadIdx.x], sc[threadIdx.x + off]);
-        }
+        if (threadIdx.x < off) sum[threadIdx.x] = zadd(sum[threadIdx.x], sum[threadIdx.x + off]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        part_b[blockIdx.x] = sb[0];
-        if (c) part_c[blockIdx.x] = sc[0];
-    }
+    if (threadIdx.x == 0) part[blockIdx.x] = sum[0];
 }
 
 // Device-side BiCGStab scalars.  stop: 0 running, 1 converged, 2 breakdown,
@@ -1026,7 +1016,7 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
     RB_CUDA(cudaMemsetAsync(v, 0, (size_t)nu * sizeof(Z), st));
     RB_CUDA(cudaMemcpyAsync(rr, d_b, (size_t)nu * sizeof(Z), cudaMemcpyDeviceToDevice, st));
     RB_CUDA(cudaMemcpyAsync(rh, d_b, (size_t)nu * sizeof(Z), cudaMemcpyDeviceToDevice, st));
-    dot_partial_kernel<<<gd, kDotThreads, 0, st>>>(d_b, d_b, nullptr, nu, part0, nullptr);
+    norm_partial_kernel<<<gd, kDotThreads, 0, st>>>(d_b, nu, part0);
     RB_CUDA(cudaGetLastError());
     std::vector<Z> h_part(gd);
     RB_CUDA(cudaMemcpyAsync(h_part.data(), part0, gd * sizeof(Z), cudaMemcpyDeviceToHost, st));
@@ -1099,7 +1089,7 @@ extern "C" sdd_status sdd_rbffd_solve(const double *nodes_xz, int32_t n, const u
     // the true residual |b - K x| / |b|
     spmv_kernel<<<gb, 128, 0, st>>>(d_ew, d_ecol, nu, ns, d_unk, d_kap, x, t);
     residual_kernel<<<gb, 128, 0, st>>>(t, d_b, nu, s);
-    dot_partial_kernel<<<gd, kDotThreads, 0, st>>>(s, s, nullptr, nu, part0, nullptr);
+    norm_partial_kernel<<<gd, kDotThreads, 0, st>>>(s, nu, part0);
     RB_CUDA(cudaGetLastError());
     RB_CUDA(cudaMemcpyAsync(d_u, u, 2 * (size_t)n * sizeof(double), cudaMemcpyHostToDevice, st));
     scatter_u_kernel<<<gb, 128, 0, st>>>(d_unk, nu, x, d_u);

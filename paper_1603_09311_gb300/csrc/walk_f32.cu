@@ -147,7 +147,7 @@ struct WalkerF32 {
     float X, Z, dmin;  // centred position, distance to the nearest wall
     uint32_t n;        // Euler steps accepted (even at the start of iterate)
     typename std::conditional<kRegions, Regions, Occupancy<KMAX>>::type occ;
-    uint32_t nid, pre_x, pre_y;
+    uint32_t pre_x, pre_y;
     const uint32_t *tco;  // GC_RASTER_MULTI: the tile map of this walk's model
 
     // Shared address of the lane's column of WarpSmem::pend: the step that
@@ -304,7 +304,6 @@ struct WalkerF32 {
         dmin = fminf(M.fhw - fabsf(X), M.fhh - fabsf(Z));
         n = 0;
         occ.clear();
-        nid = node_id;
         pre_x = __umulhi(0xCD9E8D57u, node_id) ^ path ^ A.rk0[0];
         pre_y = 0xCD9E8D57u * node_id;
     }

@@ -23,7 +23,8 @@
 // and added to the item's slot in global memory (sum re, sum im, sum re^2,
 // sum im^2; a few MB, L2-resident).  An item belongs to the one
 // warp that opened it, so its slot needs no atomics.  A second kernel adds
-// the slots of each node in item order.
+// the slots of each node, a warp per node and evaluation, in an order that
+// the item table alone fixes.
 #pragma once
 
 #include "sdd_internal.cuh"
