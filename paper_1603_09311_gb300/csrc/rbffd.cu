@@ -339,9 +339,17 @@ constexpr int kTries = 300;
 
 // Barrier of all CTAs of the (cooperative) launch, in two halves.  A wait that
 // runs out sets the top bit of the counter while arrivals are missing, by
-// compare-and-swap on the count it has just read: once all have arrived nobody
-// can fail the barrier any more, and until then nobody has passed it, so every
-// CTA leaves this barrier with the same answer.
+// compare-and-swap on the count read: once all have arrived nobody can fail the
+// barrier any more, and until then nobody has passed it, so every CTA leaves
+// this barrier with the same answer.  (Out of line: in the wait's loop it took
+// 0.25 us of an iteration's 26.)
+__device__ __noinline__ void give_up(unsigned *bar, unsigned v, unsigned epoch) {
+    while (!(v & kBarrierFail) && v < epoch) {
+        const unsigned seen = atomicCAS(bar, v, v | kBarrierFail);
+        if (seen == v) return;
+        v = seen;
+    }
+}
 __device__ __forceinline__ void grid_arrive(unsigned *bar, unsigned &epoch) {
     epoch += gridDim.x;
     __syncthreads();
@@ -354,10 +362,7 @@ __device__ __forceinline__ bool grid_wait(unsigned *bar, unsigned epoch, int *ok
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
             if ((v & kBarrierFail) || v >= epoch) break;
-            if (clock64() - t0 > kBarrierCycles && atomicCAS(bar, v, v | kBarrierFail) == v) {
-                v |= kBarrierFail;
-                break;
-            }
+            if (clock64() - t0 > kBarrierCycles) give_up(bar, v, epoch);
         }
         *ok = (v & kBarrierFail) == 0;
     }
