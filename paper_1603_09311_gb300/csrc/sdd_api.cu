@@ -986,14 +986,15 @@ namespace {
 // The current context's id, which no other context of the process ever has: a
 // device that other code has reset comes back with another one.
 cudaError_t context_id(unsigned long long *id) {
-    void *f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q);
-    if (e != cudaSuccess) return e;
-    if (q != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
-    return reinterpret_cast<CUresult (*)(CUcontext, unsigned long long *)>(f)(nullptr, id) == CUDA_SUCCESS
-               ? cudaSuccess
-               : cudaErrorDeviceUninitialized;
+    using Get = CUresult (*)(CUcontext, unsigned long long *);
+    static const Get get = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q);
+        return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<Get>(f) : nullptr;
+    }();
+    if (!get) return cudaErrorNotSupported;
+    return get(nullptr, id) == CUDA_SUCCESS ? cudaSuccess : cudaErrorDeviceUninitialized;
 }
 }  // namespace
 
