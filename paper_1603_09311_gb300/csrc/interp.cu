@@ -244,7 +244,7 @@ __global__ void linear_kernel(const double *sk, int nk, const double *v, const d
 // of the columns that reach the segment are formed once, a thread each, then
 // every thread adds up a component.  With a thread for each target and
 // component and all knots in each sum, 1025 targets x 32 components x 257 knots
-// took 0.35 ms.
+// took 0.35 ms; 0.03 ms so, behind 0.04 ms for the columns.
 constexpr int kSplineThreads = 64;
 constexpr int kWeights = 512;
 __global__ void __launch_bounds__(kSplineThreads)
