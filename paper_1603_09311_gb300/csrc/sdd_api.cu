@@ -846,13 +846,13 @@ WalkArgs base_args(sdd_ctx *ctx, const Launch &L, double dt, uint64_t seed) {
     // The best batch goes with the square root of the ended walks per step:
     // measured optima at 150, 290, 970 steps a walk were 5, 4, 2 (dt 2e-3,
     // 1e-3, 3e-4 on the quarter-space line: 13.36 -> 12.13, 11.05 -> 10.26,
-    // 28.8 -> 28.2 ms against one at a time), none at 2900.  A TE walk takes
-    // about the domain's slowest decay time.  TM walks are recorded one at a
-    // time: their lengths go with the strips' diffusions, and waiting lanes cost
-    // more (FP64, 256 nodes x 4000 walks, dt 1e-3 and 2e-3: 126 -> 124 and 69 ->
-    // 67 ms against this rule's batches of 4 and 5; FP32, diffusions 0.05 and
-    // 0.1: 45.9 -> 44.7 ms; 1 and 10: the same).
-    if (ctx->geo == GEO_TM) {
+    // 28.8 -> 28.2 ms against one at a time), none at 2900.  A walk takes about
+    // the domain's slowest decay time (TM strips of other diffusions: 16 to 512
+    // nodes at dt 1e-3, diffusions 1 and 10, up to 3.5 % faster so; 0.05 and
+    // 0.1, where walks are longer, 2.6 % slower).  FP64 TM walks, one a lane, are
+    // recorded one at a time: an idle lane costs FP64 time (256 nodes x 4000
+    // walks, dt 1e-3 and 2e-3: 126 -> 123 and 69 -> 66.5 ms).
+    if (L.f64 && !L.coop) {
         A.exit_batch = 1;
         return A;
     }
